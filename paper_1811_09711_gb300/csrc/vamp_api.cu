@@ -31,6 +31,7 @@ struct vamp_ctx {
     int64_t gen_batch = 1 << 20;
     int sm_count = 0;
     int tile = 1;              // channels per staged tile
+    int dshift = 0;            // log2 of the d-value copies in shared memory
     size_t smem_pass = 0;      // dynamic shared memory of the integration pass kernel
     size_t smem_gen = 0;       // ... of the generation pass kernel
     const PassVariant* var = nullptr;  // pass kernels in use
@@ -125,6 +126,7 @@ vamp::PassArgs pass_args(const vamp_ctx* c, uint32_t field)
     A.field = field;
     A.tile = c->tile;
     A.ntiles = (c->K + c->tile - 1) / c->tile;
+    A.dshift = c->dshift;
     return A;
 }
 
@@ -137,22 +139,10 @@ std::mutex g_tune_mu;
 std::map<std::tuple<int, int, int, int, int, int, int>, const PassVariant*> g_tuned;
 
 // Tile and shared memory of one candidate (its CTAs-per-SM budget).
-struct VariantShape {
-    int tile;
-    size_t smem_pass, smem_gen;
-};
-
-VariantShape shape_of(const vamp_ctx* c, const PassVariant* v)
+vamp::TilePlan shape_of(const vamp_ctx* c, const PassVariant* v)
 {
-    VariantShape s{};
-    if (v->uni) {
-        s.tile = 1;
-        s.smem_pass = vamp::union_pass_smem(c->prm, *v, 0);
-        s.smem_gen = vamp::union_pass_smem(c->prm, *v, 1);
-        return s;
-    }
-    vamp::pass_smem_for(c->prm, c->fp32, v->minb, &s.tile, &s.smem_pass, &s.smem_gen);
-    return s;
+    if (v->uni) return vamp::TilePlan{1, 0, vamp::union_pass_smem(c->prm, *v, 0), vamp::union_pass_smem(c->prm, *v, 1)};
+    return vamp::pass_smem(c->prm, c->fp32, v->minb);
 }
 
 // Allocates the union pass's interval tables once; false (and the
@@ -205,15 +195,16 @@ vamp_status use_variant(vamp_ctx* c, const PassVariant* v)
     } else if (!v->uni && c->uni_buf) {
         union_disable(c);
     }
-    const VariantShape s = shape_of(c, v);
-    VAMP_CK(c, vamp::ensure_smem(v->fn[0], s.smem_pass));
+    const vamp::TilePlan s = shape_of(c, v);
+    VAMP_CK(c, vamp::ensure_smem(v->fn[0], s.smem_int));
     VAMP_CK(c, vamp::ensure_smem(v->fn[1], s.smem_gen));
     int b0 = 0, b1 = 0;
-    VAMP_CK(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b0, v->fn[0], vamp::PASS_THREADS, s.smem_pass));
+    VAMP_CK(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b0, v->fn[0], vamp::PASS_THREADS, s.smem_int));
     VAMP_CK(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b1, v->fn[1], vamp::PASS_THREADS, s.smem_gen));
     c->var = v;
     c->tile = s.tile;
-    c->smem_pass = s.smem_pass;
+    c->dshift = s.dshift;
+    c->smem_pass = s.smem_int;
     c->smem_gen = s.smem_gen;
     c->grid_pass = (b0 > 0 ? b0 : 1) * c->sm_count;
     c->grid_gen = (b1 > 0 ? b1 : 1) * c->sm_count;
@@ -232,15 +223,15 @@ vamp_status choose_variant(vamp_ctx* c, int64_t n_calls)
                    cand.end());
     if (cand.empty()) return fail(c, VAMP_ERR_INVALID_ARG, "no pass kernel for this shape");
     for (const PassVariant* v : cand) {
-        const VariantShape s = shape_of(c, v);
-        VAMP_CK(c, vamp::ensure_smem(v->fn[0], s.smem_pass));
+        const vamp::TilePlan s = shape_of(c, v);
+        VAMP_CK(c, vamp::ensure_smem(v->fn[0], s.smem_int));
         VAMP_CK(c, vamp::ensure_smem(v->fn[1], s.smem_gen));
     }
     auto grid_of = [&](const PassVariant* v, int mode, int* grid) -> cudaError_t {
-        const VariantShape s = shape_of(c, v);
+        const vamp::TilePlan s = shape_of(c, v);
         int b = 0;
         cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, v->fn[mode], vamp::PASS_THREADS,
-                                                                      mode ? s.smem_gen : s.smem_pass);
+                                                                      mode ? s.smem_gen : s.smem_int);
         *grid = (b > 0 ? b : 1) * c->sm_count;
         return e;
     };
@@ -272,15 +263,16 @@ vamp_status choose_variant(vamp_ctx* c, int64_t n_calls)
         for (const PassVariant* v : cand) {
             int grid = 0;
             VAMP_CK(c, grid_of(v, 0, &grid));
-            const VariantShape s = shape_of(c, v);
+            const vamp::TilePlan s = shape_of(c, v);
             vamp::PassArgs A = pass_args(c, 0x7fffffffu);
             A.tile = s.tile;
             A.ntiles = (c->K + s.tile - 1) / s.tile;
+            A.dshift = s.dshift;
             float ms_v = 0.f;
             for (int rep = 0; rep < 2; ++rep) {
                 VAMP_CK(c, vamp::launch_begin_pass(c->prm, probe, c->stream));
                 VAMP_CK(c, cudaEventRecord(e0, c->stream));
-                VAMP_CK(c, v->launch(c->prm, 0, A, grid, s.smem_pass, c->stream));
+                VAMP_CK(c, v->launch(c->prm, 0, A, grid, s.smem_int, c->stream));
                 VAMP_CK(c, cudaEventRecord(e1, c->stream));
                 VAMP_CK(c, cudaEventSynchronize(e1));
                 VAMP_CK(c, cudaEventElapsedTime(&ms_v, e0, e1));
@@ -397,10 +389,9 @@ vamp_status vamp_create(const vamp_config* cfg, void* cuda_stream, vamp_ctx** ou
     CREATE_CK(vamp::launch_derive(P, c->stream));
     CREATE_CK(cudaStreamSynchronize(c->stream));
     {
-        vamp::pass_smem(P, c->fp32, &c->tile, &c->smem_pass, &c->smem_gen);
         int maxsm = 0;
         CREATE_CK(cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->dev));
-        if ((int)c->smem_pass > maxsm) { st = fail(c, VAMP_ERR_INVALID_ARG, "grid too large for shared memory"); goto create_fail; }
+        if ((int)vamp::pass_smem(P, c->fp32).smem_int > maxsm) { st = fail(c, VAMP_ERR_INVALID_ARG, "grid too large for shared memory"); goto create_fail; }
         CREATE_CK(cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->dev));
         // until the first pass picks by timing: the first candidate (the
         // shape-specialised kernel if there is one)

@@ -114,13 +114,10 @@ vamp_status apply_shape(vamp_batch* b, int budget_kb, int64_t item_calls)
     b->minb = budget_kb > 80 ? 2 : 3;  // 112 KB: two CTAs per SM; 72 KB: three
     size_t smem = 0;
     for (int i = 0; i < b->n; ++i) {
-        const size_t ds = (size_t)b->d[i] * b->nb[i] * 8;
-        const size_t fixed = vamp::SMEM_HEAD + vamp::PARAMS_SLOT + ds;
-        long t = budget > fixed ? (long)((budget - fixed) / (2 * b->S[i])) : 1;
-        if (t < 1) t = 1;
-        if (t > b->K[i]) t = b->K[i];
-        b->tiles[i] = (int)t;
-        smem = std::max(smem, fixed + 2 * (size_t)t * b->S[i]);
+        const vamp::TilePlan plan =
+            vamp::plan_tiles(b->S[i], b->K[i], b->d[i] * b->nb[i], vamp::SMEM_HEAD + vamp::PARAMS_SLOT, budget);
+        b->tiles[i] = plan.tile | plan.dshift << 24;
+        smem = std::max(smem, plan.smem_int);
     }
     int maxsm = 0;
     BCK(b, cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, b->dev));

@@ -33,11 +33,11 @@ __device__ __forceinline__ bool run_item(const MultiArgs& M, const Params& P, Sm
     constexpr int B = PASS_THREADS * CPT;
     const int tid = threadIdx.x;
     const SH sh(Prec<T>::lay(P), P.d, P.n);
-    const int tile = M.tiles[inst];
+    const int tile = M.tiles[inst] & 0xffffff, dshift = M.tiles[inst] >> 24;
     const int ntiles = (P.K + tile - 1) / tile;
     const int S = sh.bytes();
     const size_t tile_bytes = (size_t)tile * S;
-    double* Ds = reinterpret_cast<double*>(buf0 + 2 * tile_bytes);
+    double* Ds = reinterpret_cast<double*>(buf0 + (ntiles > 1 ? 2 : 1) * tile_bytes);
     const int dn = P.d * P.n;
     const int64_t a = P.Pc[c] + kth * M.item_calls;
     const int64_t b = min(a + M.item_calls, (int64_t)P.Pc[c + 1]);
@@ -51,7 +51,7 @@ __device__ __forceinline__ bool run_item(const MultiArgs& M, const Params& P, Sm
         fence_proxy_async_smem();
         bulk_load(buf0 + (u & 1) * tile_bytes, lk + (size_t)t * tile_bytes, (uint32_t)(cnt * S), &H.bar[u & 1]);
     };
-    for (int q = tid; q < dn; q += PASS_THREADS) Ds[q] = 0.0;
+    for (int q = tid; q < dn << dshift; q += PASS_THREADS) Ds[q] = 0.0;
     __syncthreads();
     if (tid == 0) {
         issue(0);
@@ -93,7 +93,7 @@ __device__ __forceinline__ bool run_item(const MultiArgs& M, const Params& P, Sm
             }
             ++u;
         }
-        phase_c_int<T, CPT>(sh, C, sft, Ds, s1, s2, wm, bad,
+        phase_c_int<T, CPT>(sh, C, sft, Ds, dshift, s1, s2, wm, bad,
                             (SH::kStrat && P.stratified) ? CellSums{P.cellsum, base - P.Pc[c], P.spc[c], P.coff[c]}
                                                          : CellSums{nullptr, 0, 1, 0});
     }
@@ -105,7 +105,7 @@ __device__ __forceinline__ bool run_item(const MultiArgs& M, const Params& P, Sm
         pp.done0 += 1u;
         pp.done1 += ntiles > 1 ? 1u : 0u;
     }
-    flush_segment(P, H, c, dn, Ds, s1, s2);
+    flush_segment(P, H, c, dn, Ds, dshift, s1, s2);
     block_max_to(H, wm, &P.sc->wmax_bits);
     return true;
 }

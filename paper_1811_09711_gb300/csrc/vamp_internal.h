@@ -28,6 +28,7 @@ struct PassArgs {
     uint32_t field;
     int tile;          // channels per staged tile
     int ntiles;        // ceil(K / tile)
+    int dshift;        // log2 of the copies of the d-values in shared memory
     int rec_bytes;
     int64_t batch;
     int64_t chunk;
@@ -101,10 +102,19 @@ void bind_arena(Params& P, unsigned char* base, const Arena& A);  // sets every 
 // Copies headers and peak records into the arena (async on s).
 cudaError_t upload_setup(const Params& P, const Setup& S, cudaStream_t s);
 
-// Tile and shared-memory size of the pass kernel: two CTAs per SM
-// (TILE_BUDGET), or `minb` CTAs per SM of the current device.
-void pass_smem(const Params& P, int fp32, int* tile, size_t* smem_int, size_t* smem_gen);
-void pass_smem_for(const Params& P, int fp32, int minb, int* tile, size_t* smem_int, size_t* smem_gen);
+// Shared-memory layout of a staged-tile pass kernel: channels per tile, log2
+// of the copies of the d-values, bytes of the integration and generation form.
+// One tile that holds every channel takes one buffer, several take two.
+struct TilePlan {
+    int tile, dshift;
+    size_t smem_int, smem_gen;
+};
+// For K lookup blocks of S bytes and dn = d n bins beside `fixed` bytes in a
+// budget (see vamp_setup.cu for how the d-value copies are chosen).
+TilePlan plan_tiles(size_t S, int K, int dn, size_t fixed, size_t budget);
+// The pass kernel's, at two CTAs per SM (TILE_BUDGET) or `minb` CTAs per SM
+// of the current device.
+TilePlan pass_smem(const Params& P, int fp32, int minb = 2);
 // Candidate kernels for a shape: exact (D, NB) matches first, then generic;
 // with the channel count K given (K > 0) and union_fits, the union kernels
 // after them (exact shape first).
@@ -126,7 +136,7 @@ struct BatchCtl {
 };
 struct MultiArgs {
     const Params* inst;          // [n] instance parameters
-    const int* tiles;            // [n] channels per staged tile
+    const int* tiles;            // [n] channels per staged tile (low 24 bits) | d-value copies (log2) << 24
     const int* combine_from;     // [n]
     const int64_t* ncalls;       // [n] calls requested this iteration
     const uint32_t* iter;        // [n] iteration index (random stream) of each instance

@@ -103,10 +103,9 @@ extern "C" vamp_status vamp_sample_pass_static(const vamp_config* cfg, const dou
         put_msg(err_msg, err_len, msg);
         return VAMP_ERR_INVALID_ARG;
     }
-    int tile = 1;
-    size_t smem = 0, smem_gen = 0;
     const std::vector<const vamp::PassVariant*> cand = vamp::pass_candidates(fp32, d, n);
-    vamp::pass_smem_for(pr, fp32, cand.empty() ? 2 : cand[0]->minb, &tile, &smem, &smem_gen);
+    const vamp::TilePlan plan = vamp::pass_smem(pr, fp32, cand.empty() ? 2 : cand[0]->minb);
+    const size_t smem = plan.smem_int;
 
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -144,8 +143,9 @@ extern "C" vamp_status vamp_sample_pass_static(const vamp_config* cfg, const dou
     if (e == cudaSuccess) {
         vamp::PassArgs A{};
         A.field = iteration;
-        A.tile = tile;
-        A.ntiles = (K + tile - 1) / tile;
+        A.tile = plan.tile;
+        A.ntiles = (K + plan.tile - 1) / plan.tile;
+        A.dshift = plan.dshift;
         e = var->launch(pr, 0, A, (bps > 0 ? bps : 1) * sms, smem, stream);
     }
     if (e == cudaSuccess) e = vamp::launch_finish_pass(pr, 0, stream);

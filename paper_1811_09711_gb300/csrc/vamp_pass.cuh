@@ -67,9 +67,24 @@ struct CellSums {
     int64_t coff;    // first cell of the channel
 };
 
+// Calls of an integration batch: warp w takes the 32 CPT calls from 32 CPT w
+// on, so that a short batch leaves whole warps without calls, and they skip
+// it (the 1e4-call pass of a d = 4 problem has 33 calls per CTA).
+template <int CPT>
+__device__ __forceinline__ int warp_first()
+{
+    return (int)(threadIdx.x >> 5) * (32 * CPT);
+}
+template <int CPT>
+__device__ __forceinline__ int call_of(int q)
+{
+    return warp_first<CPT>() + q * 32 + (int)(threadIdx.x & 31);
+}
+
 // Phase A: Philox words, channel, forward map on the channel's grid, own
 // term of g(p), Gaussian exponent sum; the integrand when peaks are not the
-// channels' maps.  Call q of this thread is base + q*PASS_THREADS + tid.
+// channels' maps.  Call q of this thread is base + call_of(q) (integration)
+// or base + q*PASS_THREADS + tid (generation, whose records are in that order).
 template <typename T, int MODE, int CPT, class SH>
 __device__ __forceinline__ void phase_a(const Params& P, const SH& sh, uint32_t field, int64_t base, int64_t end,
                                         int cseg, Calls<T, CPT, SH::DM>& C)
@@ -79,7 +94,7 @@ __device__ __forceinline__ void phase_a(const Params& P, const SH& sh, uint32_t 
     const int tid = threadIdx.x;
 #pragma unroll
     for (int q = 0; q < CPT; ++q) {
-        const int64_t i = base + (int64_t)q * PASS_THREADS + tid;
+        const int64_t i = base + (MODE == 0 ? call_of<CPT>(q) : q * PASS_THREADS + tid);
         C.valid[q] = i < end;
         uint32_t X[DM + 4];
         call_words<DM + 4>(P, (uint32_t)(C.valid[q] ? i : base), field, MODE == 0 ? d : d + 2, X);
@@ -160,19 +175,21 @@ __device__ __forceinline__ uint32_t pick(const uint32_t (&a)[W], int i)
 
 // Phase C of an integration batch: shifted sums, max weight and the d-values
 // (Eq. 15) of the segment's channel in shared memory (FP64 atomics, which
-// retry on collisions).  Unless the shape has many bins per axis (a lane's
-// bins then rarely collide), lane l adds its d terms in the rotated axis
-// order l, l+1, ... (mod d), so that at any step the lanes of a warp hit
-// different rows.
+// retry on collisions), in 2^dshift copies (plan_tiles).  Unless the shape has
+// many bins per axis (a lane's bins then rarely collide), lane l adds its d
+// terms in the rotated axis order l, l+1, ... (mod d), so that at any step the
+// lanes of a warp hit different rows, and lanes that share a row (l, l+d, ...)
+// different copies.
 template <typename T, int CPT, class SH>
 __device__ __forceinline__ void phase_c_int(const SH& sh, const Calls<T, CPT, SH::DM>& C, double sft, double* Ds,
-                                            double& s1, double& s2, double& wm, bool& bad,
+                                            int dshift, double& s1, double& s2, double& wm, bool& bad,
                                             const CellSums cs = CellSums{nullptr, 0, 1, 0})
 {
     constexpr int DM = SH::DM;
-    const int d = sh.d(), n = sh.n();
+    const int d = sh.d(), n = sh.n(), lane = threadIdx.x & 31;
     constexpr bool kRotate = !(SH::kN && SH::NBC >= 64);
-    const int rot = kRotate ? (threadIdx.x & 31) % d : 0;
+    const int rot = kRotate ? lane % d : 0;
+    double* Dl = Ds + ((kRotate ? lane / d : lane) & ((1 << dshift) - 1));
 #pragma unroll
     for (int q = 0; q < CPT; ++q) {
         if (!C.valid[q]) continue;
@@ -182,20 +199,20 @@ __device__ __forceinline__ void phase_c_int(const SH& sh, const Calls<T, CPT, SH
         s1 += dv;
         s2 += dv * dv;
         if (cs.sum)  // stratified: the sum of the call's cell
-            atomicAdd(&cs.sum[cs.coff + (cs.l0 + q * PASS_THREADS + (int)threadIdx.x) / cs.spc], dv);
+            atomicAdd(&cs.sum[cs.coff + (cs.l0 + call_of<CPT>(q)) / cs.spc], dv);
         wm = fmax(wm, fabs(w));  // signed integrands: w_max bounds |w|
         const double w2 = w * w;
 #pragma unroll
         for (int s = 0; s < DM; ++s) {
             if (sh.has(s)) {
+                int k = s;
+                uint32_t v = C.jp[q][s >> 2];
                 if (kRotate) {
-                    int k = s + rot;
+                    k = s + rot;
                     if (k >= d) k -= d;
-                    const int j = (pick(C.jp[q], k >> 2) >> (8 * (k & 3))) & 0xff;
-                    atomicAdd(&Ds[k * n + j], w2);
-                } else {
-                    atomicAdd(&Ds[s * n + ((C.jp[q][s >> 2] >> (8 * (s & 3))) & 0xff)], w2);
+                    v = pick(C.jp[q], k >> 2);
                 }
+                atomicAdd(&Dl[(k * n + (int)((v >> (8 * (k & 3))) & 0xff)) << dshift], w2);
             }
         }
     }
@@ -257,8 +274,8 @@ __device__ __forceinline__ void phase_c_gen(const Params& P, const PassArgs& A, 
 }
 
 // Flush of a segment: block sums of (s1, s2) and the d-values to global.
-__device__ __forceinline__ void flush_segment(const Params& P, SmemHead& H, int cseg, int dn, double* Ds, double s1,
-                                              double s2)
+__device__ __forceinline__ void flush_segment(const Params& P, SmemHead& H, int cseg, int dn, double* Ds,
+                                              int dshift, double s1, double s2)
 {
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     s1 = warp_sum(s1);
@@ -273,7 +290,8 @@ __device__ __forceinline__ void flush_segment(const Params& P, SmemHead& H, int 
     }
     double* Dg = P.D + (size_t)cseg * dn;
     for (int q = tid; q < dn; q += PASS_THREADS) {
-        const double v = Ds[q];
+        double v = 0.0;
+        for (int r = 0; r < 1 << dshift; ++r) v += Ds[(q << dshift) + ((r + tid) & ((1 << dshift) - 1))];
         if (v != 0.0) atomicAdd(&Dg[q], v);
     }
     __syncthreads();
@@ -304,22 +322,24 @@ __global__ void __launch_bounds__(PASS_THREADS, MINB) k_pass(Params P, PassArgs 
     const SH sh(Prec<T>::lay(P), P.d, P.n);
     const int S = sh.bytes();
     const size_t tile_bytes = (size_t)A.tile * S;
-    double* Ds = reinterpret_cast<double*>(buf0 + 2 * tile_bytes);
+    const size_t tiles_bytes = (A.ntiles > 1 ? 2 : 1) * tile_bytes;
+    double* Ds = reinterpret_cast<double*>(buf0 + tiles_bytes);
     const int d = sh.d(), n = sh.n(), dn = d * n, K = P.K;
+    int dshift = A.dshift;
     const int tid = threadIdx.x;
     constexpr int B = PASS_THREADS * CPT;
     const unsigned char* lk = Prec<T>::lk(P);
     // FP64: the power-law Jacobian 0.2 p_k^(-4/5) of each coordinate of this
     // thread's call, computed once per call instead of once per channel that
     // maps k (after the tiles and the d-values; DMAX x PASS_THREADS doubles
-    // are reserved by smem_for_budget)
+    // are reserved by pass_smem)
     constexpr bool kPW = sizeof(T) == 8 && CPT == 1;
     T* pwS = nullptr;
     if constexpr (kPW) {
-        // used only where the launch reserved the space (see smem_for_budget)
+        // used only where the launch reserved the space (see pass_smem)
         unsigned dsm = 0;
         asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dsm));
-        const size_t off = SMEM_HEAD + 2 * tile_bytes + (MODE == 0 ? (size_t)dn * 8 : 0);
+        const size_t off = SMEM_HEAD + tiles_bytes + (MODE == 0 ? (size_t)(dn << A.dshift) * 8 : 0);
         if ((size_t)dsm >= off + (size_t)DM * PASS_THREADS * sizeof(T))
             pwS = reinterpret_cast<T*>(smem + off);
     }
@@ -329,8 +349,10 @@ __global__ void __launch_bounds__(PASS_THREADS, MINB) k_pass(Params P, PassArgs 
     int64_t nbatch = 0;
     if (MODE == 0) {
         const int64_t N = P.sc->n_total;
-        r0 = N * blockIdx.x / gridDim.x;
-        r1 = N * (blockIdx.x + 1) / gridDim.x;
+        // whole warps of calls, so that a small pass has few half-empty ones
+        r0 = (N * blockIdx.x / gridDim.x) & ~int64_t(31);
+        r1 = blockIdx.x + 1 < gridDim.x ? (N * (blockIdx.x + 1) / gridDim.x) & ~int64_t(31) : N;
+        if (r1 - r0 < (int64_t)n << dshift) dshift = 0;  // fewer d-value adds than words to clear and sum
         int64_t i = r0;
         while (i < r1) {
             const int c = find_channel(P.Pc, K, i);
@@ -385,7 +407,7 @@ __global__ void __launch_bounds__(PASS_THREADS, MINB) k_pass(Params P, PassArgs 
                 cseg = find_channel(P.Pc, K, i0);
                 seg_end = min(r1, P.Pc[cseg + 1]);
                 sft = P.shift[cseg];
-                for (int q = tid; q < dn; q += PASS_THREADS) Ds[q] = 0.0;
+                for (int q = tid; q < dn << dshift; q += PASS_THREADS) Ds[q] = 0.0;
                 s1 = s2 = 0.0;
                 __syncthreads();
             }
@@ -398,9 +420,10 @@ __global__ void __launch_bounds__(PASS_THREADS, MINB) k_pass(Params P, PassArgs 
 
         // ---- phase A: own channel forward map, integrand --------------------
         Calls<T, CPT, DM> C;
-        phase_a<T, MODE, CPT>(P, sh, A.field, base, end, cseg, C);
+        const bool live = MODE == 1 || base + warp_first<CPT>() < end;  // some call of this warp
+        if (live) phase_a<T, MODE, CPT>(P, sh, A.field, base, end, cseg, C);
         if constexpr (kPW) {
-            if (pwS) {
+            if (live && pwS) {
 #pragma unroll
                 for (int k = 0; k < DM; ++k) {
                     if (sh.has(k)) {
@@ -422,7 +445,7 @@ __global__ void __launch_bounds__(PASS_THREADS, MINB) k_pass(Params P, PassArgs 
                     H.abort = 1;
                 }
             }
-            if (!H.abort)
+            if (live && !H.abort)
                 tile_compute<T, MODE, CPT>(P, sh, buf0 + b * tile_bytes, t, A.tile, cseg, C, pwS ? pwS + tid : nullptr);
             __syncthreads();
             if (H.abort) goto drain;
@@ -435,14 +458,15 @@ __global__ void __launch_bounds__(PASS_THREADS, MINB) k_pass(Params P, PassArgs 
 
         // ---- phase C: weights and accumulation ------------------------------
         if (MODE == 0) {
-            phase_c_int<T, CPT>(sh, C, sft, Ds, s1, s2, wm, bad,
-                                (SH::kStrat && P.stratified)
-                                    ? CellSums{P.cellsum, base - P.Pc[cseg], P.spc[cseg], P.coff[cseg]}
-                                    : CellSums{nullptr, 0, 1, 0});
+            if (live)
+                phase_c_int<T, CPT>(sh, C, sft, Ds, dshift, s1, s2, wm, bad,
+                                    (SH::kStrat && P.stratified)
+                                        ? CellSums{P.cellsum, base - P.Pc[cseg], P.spc[cseg], P.coff[cseg]}
+                                        : CellSums{nullptr, 0, 1, 0});
             i0 = end;
             if (i0 >= seg_end) {
                 // end of the segment: flush its sums and d-values
-                flush_segment(P, H, cseg, dn, Ds, s1, s2);
+                flush_segment(P, H, cseg, dn, Ds, dshift, s1, s2);
                 s1 = s2 = 0.0;
             }
         } else {

@@ -68,7 +68,7 @@ struct Req {
     long long* offsets = nullptr;
     const vamp::PassVariant* var = nullptr;
     int tile = 1, grid_gen = 0;
-    size_t smem_int = 0, smem_gen = 0;
+    size_t smem_gen = 0;
     int64_t chunk = 0, nchunks = 0, gen_batch = 0;
     int lane = -1;             // index into the server's lanes
     cudaStream_t stream = nullptr;
@@ -237,7 +237,9 @@ vamp_status admit(vamp_server* s, Req* r)
     if (e == cudaSuccess) e = cudaEventRecord(r->ev, r->stream);  // setup done (polled)
     if (e != cudaSuccess) return VAMP_ERR_CUDA;
     // generation kernel of this shape
-    vamp::pass_smem_for(P, s->fp32, r->var->minb, &r->tile, &r->smem_int, &r->smem_gen);
+    const vamp::TilePlan plan = vamp::pass_smem(P, s->fp32, r->var->minb);
+    r->tile = plan.tile;
+    r->smem_gen = plan.smem_gen;
     e = vamp::ensure_smem(r->var->fn[1], r->smem_gen);
     int bps = 0;
     if (e == cudaSuccess)
@@ -303,13 +305,10 @@ vamp_status tick_launch(vamp_server* s, const std::vector<Req*>& ints)
         Req* r = ints[i];
         const Params& P = r->P;
         const size_t S = (size_t)(s->fp32 ? P.lay32.bytes : P.lay64.bytes);
-        const size_t ds = (size_t)P.d * P.n * 8;
-        const size_t fixed = vamp::SMEM_HEAD + vamp::PARAMS_SLOT + ds;
-        long t = s->tick_budget > fixed ? (long)((s->tick_budget - fixed) / (2 * S)) : 1;
-        t = std::max(1L, std::min(t, (long)P.K));
-        smem = std::max(smem, fixed + 2 * (size_t)t * S);
+        const vamp::TilePlan plan = vamp::plan_tiles(S, P.K, P.d * P.n, vamp::SMEM_HEAD + vamp::PARAMS_SLOT, s->tick_budget);
+        smem = std::max(smem, plan.smem_int);
         s->h_inst[i] = P;
-        s->h_tiles[i] = (int)t;
+        s->h_tiles[i] = plan.tile | plan.dshift << 24;
         s->h_comb[i] = r->cfg.combine_from;
         s->h_ncalls[i] = r->calls;
         s->h_iter[i] = (uint32_t)r->it_done;

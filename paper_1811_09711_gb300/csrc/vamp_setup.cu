@@ -5,6 +5,7 @@
 #include "vamp_device.cuh"
 #include "vamp_internal.h"
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -299,37 +300,31 @@ cudaError_t upload_setup(const Params& P, const Setup& S, cudaStream_t s)
     return e;
 }
 
-namespace {
-void smem_for_budget(const Params& P, int fp32, size_t budget, int* tile, size_t* smem_int, size_t* smem_gen)
+// D-value copies: the lanes of a warp that add to the same axis at a step use
+// different ones, so that calls of one bin rarely meet at one word (an FP64
+// add in shared memory is a compare-and-swap loop: a d = 4, n = 20 pass went
+// through it 36 times per add with one copy).  Every segment clears and sums
+// all copies, so they are kept below 8 KB: with 32 KB the small passes and the
+// 32-problem batch lost more than they gained (8.65 -> 9.99 ms).
+TilePlan plan_tiles(size_t S, int K, int dn, size_t fixed, size_t budget)
+{
+    const size_t most = 8 * 1024, one = (size_t)dn * 8;
+    int ds = 5;
+    while (ds > 0 && ((one << ds) > most || fixed + 2 * S + (one << ds) > budget)) --ds;
+    const size_t d = one << ds;
+    const size_t room = budget > fixed + d ? budget - fixed - d : 0;
+    TilePlan p{};
+    p.dshift = ds;
+    p.tile = (size_t)K * S <= room ? K : (int)std::max<size_t>(1, std::min<size_t>((size_t)K, room / (2 * S)));
+    const size_t tiles = (size_t)(p.tile < K ? 2 : 1) * p.tile * S;
+    p.smem_int = fixed + tiles + d;
+    p.smem_gen = fixed + tiles;
+    return p;
+}
+
+TilePlan pass_smem(const Params& P, int fp32, int minb)
 {
     const size_t S = (size_t)(fp32 ? P.lay32.bytes : P.lay64.bytes);
-    const size_t ds = (size_t)P.d * P.n * 8;
-    // FP64: each thread's power-law Jacobians of its call, one per coordinate,
-    // where they fit beside one tile in a block's largest shared memory (the
-    // kernel computes them per channel otherwise)
-    size_t pw = fp32 ? 0 : (size_t)DMAX * PASS_THREADS * 8;
-    int dev = 0, maxsm = 0;
-    if (pw && cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
-        SMEM_HEAD + 2 * S + ds + pw > (size_t)maxsm)
-        pw = 0;
-    const size_t fixed = SMEM_HEAD + ds + pw;
-    long t = budget > fixed ? (long)((budget - fixed) / (2 * S)) : 1;
-    if (t < 1) t = 1;
-    if (t > P.K) t = P.K;
-    *tile = (int)t;
-    *smem_int = SMEM_HEAD + 2 * (size_t)t * S + ds + pw;
-    *smem_gen = SMEM_HEAD + 2 * (size_t)t * S + pw;
-}
-}  // namespace
-
-void pass_smem(const Params& P, int fp32, int* tile, size_t* smem_int, size_t* smem_gen)
-{
-    smem_for_budget(P, fp32, TILE_BUDGET, tile, smem_int, smem_gen);
-}
-
-void pass_smem_for(const Params& P, int fp32, int minb, int* tile, size_t* smem_int, size_t* smem_gen)
-{
     // per-CTA share of the SM's shared memory, less the per-CTA reservation
     int dev = 0, per_sm = 0, reserved = 0;
     size_t budget = TILE_BUDGET;
@@ -337,7 +332,16 @@ void pass_smem_for(const Params& P, int fp32, int minb, int* tile, size_t* smem_
         cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) == cudaSuccess)
         budget = std::min(budget, (size_t)(per_sm / minb - reserved));
-    smem_for_budget(P, fp32, budget, tile, smem_int, smem_gen);
+    // FP64: each thread's power-law Jacobians of its call, one per coordinate,
+    // where they fit beside one tile in a block's largest shared memory (the
+    // kernel computes them per channel otherwise)
+    size_t pw = fp32 ? 0 : (size_t)DMAX * PASS_THREADS * 8;
+    int maxsm = 0;
+    if (pw && cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
+        SMEM_HEAD + 2 * S + (size_t)P.d * P.n * 8 + pw > (size_t)maxsm)
+        pw = 0;
+    return plan_tiles(S, P.K, P.d * P.n, SMEM_HEAD + pw, budget);
 }
 
 std::vector<const PassVariant*> pass_candidates(int fp32, int d, int n, int stratified, int K)

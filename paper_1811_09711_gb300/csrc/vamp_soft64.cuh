@@ -1,0 +1,267 @@
+// vamp_soft64.cuh -- products of positive numbers with 64-bit mantissas on the
+// integer pipe, for the FP64 form of the channel loop (Eq. 30).
+//
+// Why: the FP64 pipe of sm_103a retires 1.7 lanes per SM and cycle
+// (vamp_measure_peaks), about 1/75 of the 32-bit lane rate, and the FP64
+// channel loop is products all the way: d bin densities, the Jacobians, the
+// peak's factors.  A product of two 64-bit mantissas is three 32 x 32 -> 64
+// multiplies and a few adds, so a factor costs about eight issue slots
+// instead of the 75 its DMUL occupies, and truncates at 2^-62 instead of
+// rounding at 2^-53.
+//
+// A number is m 2^e with m > 0.  "Normalised" means bit 63 of m is set.
+// Products of normalised numbers are not renormalised at once: each loses at
+// most one leading bit, so four products in a row keep 60 bits.
+//
+// A packed number (one 64-bit word, the form of the density rows and of the
+// per-call tables) is the double's 53-bit significand in the high bits and its
+// biased exponent in the low eleven: value = (w & ~2047) 2^((w & 2047) - 1086).
+#pragma once
+
+#include <cstdint>
+#include <cstring>
+
+#ifdef __CUDACC__
+#define VAMP_HD __host__ __device__ __forceinline__
+#else
+#include <cmath>
+#define VAMP_HD inline
+#endif
+
+namespace vamp {
+
+struct Sf {
+    uint64_t m;
+    int e;
+};
+
+constexpr int SF_BIAS = 1086;  // exponent field of a double + 63 bits of mantissa below the leading one
+
+VAMP_HD uint64_t sf_bits(double x)
+{
+#ifdef __CUDA_ARCH__
+    return (uint64_t)__double_as_longlong(x);
+#else
+    uint64_t b;
+    std::memcpy(&b, &x, 8);
+    return b;
+#endif
+}
+
+VAMP_HD double sf_from_bits(uint64_t b)
+{
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((long long)b);
+#else
+    double x;
+    std::memcpy(&x, &b, 8);
+    return x;
+#endif
+}
+
+VAMP_HD int sf_clz(uint64_t m)
+{
+#ifdef __CUDA_ARCH__
+    return __clzll((long long)m);
+#else
+    return m ? __builtin_clzll(m) : 64;
+#endif
+}
+
+// High 64 bits of a b without the low halves' product: short of the true
+// value by at most three units of 2^-64.
+VAMP_HD uint64_t sf_mulhi(uint64_t a, uint64_t b)
+{
+    const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a, bh = (uint32_t)(b >> 32), bl = (uint32_t)b;
+    return (uint64_t)ah * bh + (((uint64_t)ah * bl) >> 32) + (((uint64_t)al * bh) >> 32);
+}
+
+VAMP_HD Sf sf_norm(Sf a)
+{
+    const int s = sf_clz(a.m);
+    return Sf{a.m << (s & 63), a.e - s};
+}
+
+VAMP_HD Sf sf_mul(Sf a, Sf b) { return Sf{sf_mulhi(a.m, b.m), a.e + b.e + 64}; }
+
+// A positive normal double (a subnormal or zero reads as its exponent's
+// smallest normal, as the FP64 inverse fifth root reads it).
+VAMP_HD Sf sf_from_double(double x)
+{
+    const uint64_t b = sf_bits(x);
+    return Sf{(b << 11) | (1ull << 63), (int)((uint32_t)(b >> 52) & 0x7ffu) - SF_BIAS};
+}
+
+// Nearest double of a normalised number; 0 below the normal range, infinity above.
+VAMP_HD double sf_to_double(Sf a)
+{
+    const int x = a.e + SF_BIAS;
+    const uint64_t r = (a.m >> 11) + ((a.m >> 10) & 1u);  // [2^52, 2^53]
+    uint64_t b = ((uint64_t)(uint32_t)(x - 1) << 52) + r;
+    b = x >= 1 ? b : 0ull;
+    b = x <= 2046 ? b : 0x7ff0000000000000ull;
+    return sf_from_bits(b);
+}
+
+VAMP_HD Sf sf_unpack(uint64_t w) { return Sf{w & ~2047ull, (int)((uint32_t)w & 2047u) - SF_BIAS}; }
+
+VAMP_HD uint64_t sf_pack_double(double x)
+{
+    const uint64_t b = sf_bits(x);
+    return (b << 11) | (1ull << 63) | ((b >> 52) & 2047u);
+}
+
+VAMP_HD double sf_unpack_double(uint64_t w) { return sf_from_bits(((w & 2047u) << 52) | ((w >> 11) & 0xFFFFFFFFFFFFFull)); }
+
+// Packs a normalised number, rounded to 53 bits (exponents beyond a double's
+// range are clamped: no table entry gets there).
+VAMP_HD uint64_t sf_pack(Sf a)
+{
+    const uint64_t r = (a.m >> 11) + ((a.m >> 10) & 1u);  // [2^52, 2^53]
+    int x = a.e + SF_BIAS + (int)(r >> 53);
+    x = x < 0 ? 0 : (x > 2047 ? 2047 : x);
+    return (r << 11) | (1ull << 63) | (uint32_t)x;
+}
+
+VAMP_HD float sf_lg2f(float v)
+{
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+#else
+    return std::log2(v);
+#endif
+}
+
+VAMP_HD float sf_ex2f(float v)
+{
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+#else
+    return std::exp2(v);
+#endif
+}
+
+VAMP_HD float sf_rcpf(float v)
+{
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+#else
+    return 1.0f / v;
+#endif
+}
+
+VAMP_HD uint32_t sf_f2u(float v)  // v >= 0, saturating
+{
+#ifdef __CUDA_ARCH__
+    return __float2uint_rz(v);
+#else
+    return v >= 4294967296.0f ? 0xffffffffu : (uint32_t)v;
+#endif
+}
+
+// c a >> 31 and c a >> 30 of a 32-bit number c and a signed a below 2^44 in size
+VAMP_HD int64_t sf_scale(uint32_t c, int64_t a, int sh)
+{
+    const uint64_t lo = (uint64_t)c * (uint32_t)a;
+    const int64_t hi = (int64_t)(int32_t)(a >> 32) * (int64_t)(uint64_t)c;
+    return (hi << (32 - sh)) + (int64_t)(lo >> sh);
+}
+
+// 1 / a of a normalised number, to about 2^-61: an FP32 reciprocal y0 of x =
+// m 2^-64 in [1/2, 1), then one step of third order (Householder's method),
+// y = y0 (1 + r + r^2) with r = 1 - x y0 taken in 63-bit fixed point (|r| <=
+// 2^-22, so the next term is below 2^-66).
+VAMP_HD Sf sf_rcp(Sf a)
+{
+    const float xf = (float)(uint32_t)(a.m >> 40) * 0x1p-24f;
+    const uint32_t y0 = sf_f2u(sf_rcpf(xf) * 0x1p31f);  // Q1.31
+    const uint64_t p = (a.m >> 32) * (uint64_t)y0 + (((a.m & 0xffffffffull) * (uint64_t)y0) >> 32);  // x y0, Q1.63
+    const int64_t r = (int64_t)((1ull << 63) - p) - 3;  // |r| < 2^43, never above the true residual
+    const int32_t rh = (int32_t)(r >> 14);
+    const int64_t c = r + (int64_t)(((int64_t)rh * rh) >> 35);  // r + r^2
+    const uint64_t y = ((uint64_t)y0 << 32) + (uint64_t)sf_scale(y0, c, 31);
+    return Sf{y, -127 - a.e};
+}
+
+// v^(-4/5) of a positive normal double, normalised, to about 2^-57.  With v = X
+// 2^(5a), X in [2^-4, 2): an FP32 seed s of X^(-1/5) in (0.87, 1.75), s^2, s^4
+// and s^5 in fixed point, the residual r = 1 - X s^5 (|r| <= 2^-20), and the
+// binomial series (1 - r)^(-4/5) = 1 + (4/5) r + (18/25) r^2 + ... cut after r^2:
+// X^(-4/5) = s^4 (1 - r)^(-4/5).
+VAMP_HD Sf sf_powm08(double v)
+{
+    const uint64_t b = sf_bits(v);
+    const uint64_t m = (b << 11) | (1ull << 63);            // v = m 2^-64 2^ex
+    const int ex = (int)((uint32_t)(b >> 52) & 0x7ffu) - 1022;
+    // ex = 5 a + h with h in -3..1
+    const int a = (int)(((uint32_t)(ex + 5003) * 52429u) >> 18) - 1000;  // floor((ex + 3) / 5), ex + 5003 < 2^14
+    const int h = ex - 5 * a;
+    const float l = sf_lg2f((float)(uint32_t)(m >> 40)) + (float)(h - 24);
+    const uint32_t s = sf_f2u(sf_ex2f(-0.2f * l) * 0x1p31f);  // Q1.31
+    const uint64_t s2 = (uint64_t)s * s;                      // Q2.62
+    const uint64_t s4 = sf_mulhi(s2, s2);                     // Q4.60
+    const uint64_t s5 = (s4 >> 32) * (uint64_t)s + (((s4 & 0xffffffffull) * (uint64_t)s) >> 32);  // Q5.59
+    const uint64_t q = sf_mulhi(m, s5);                       // X s^5 2^-h, Q5.59
+    const int64_t d = (int64_t)((1ull << (59 - h)) - q);
+    const int64_t r = (int64_t)((uint64_t)d << (3 + h));      // Q0.62, |r| < 2^43
+    // 0.8 r = r - r / 5 (the constant is 2^34 / 5), 0.72 r^2
+    const int64_t r5 = (int64_t)((uint64_t)sf_scale(3435973837u, r, 32)) >> 2;
+    const int32_t rh = (int32_t)(r >> 20);
+    const uint32_t r2 = (uint32_t)(((int64_t)rh * rh) >> 22);
+    const int64_t c = r - r5 + (int64_t)(((uint64_t)r2 * 3092376453u) >> 32);
+    const uint64_t z = s4 + (uint64_t)sf_scale((uint32_t)(s4 >> 32), c, 30) +
+                       (uint64_t)((int64_t)((int64_t)(uint32_t)s4 * (int64_t)(int32_t)(c >> 30)) >> 32);
+    return sf_norm(Sf{z, -60 - 4 * a});
+}
+
+// 2^x of a finite double |x| < 2^20, normalised, to about 2^-57: the fraction's
+// leading two bits pick 2^(i/4), the rest goes through the series of 2^t =
+// sum (t ln 2)^k / k! for t in [0, 1/4), whose terms from t^7 on (below 2^-30)
+// are summed in 32 bits.
+VAMP_HD Sf sf_exp2(double x)
+{
+    const uint64_t b = sf_bits(x);
+    const int ex = (int)((uint32_t)(b >> 52) & 0x7ffu) - 1023;
+    const uint64_t mant = (b << 11) | (1ull << 63);  // |x| = mant 2^(ex - 63)
+    // integer part and 64-bit fraction of |x|
+    int n = 0;
+    uint64_t f;
+    if (ex >= 0) {
+        n = (int)(mant >> (63 - ex));
+        f = ex < 63 ? mant << (ex + 1) : 0ull;
+    } else {
+        f = ex >= -64 ? mant >> (-1 - ex) : 0ull;
+    }
+    if (b >> 63) {  // 2^-(n + f) = 2^(-n-1) 2^(1-f)
+        n = f ? -n - 1 : -n;
+        f = 0ull - f;
+    }
+    const uint32_t i = (uint32_t)(f >> 62);
+    const uint64_t t = f & 0x3fffffffffffffffull;  // Q0.64, below 1/4
+    const uint32_t th = (uint32_t)(t >> 32);
+    // (ln 2)^k / k!: 47-bit fractions for k = 12..7, 64-bit ones for k = 6..1
+    uint32_t w = 3614u;
+    w = 62565u + (uint32_t)(((uint64_t)w * th) >> 32);
+    w = 992891u + (uint32_t)(((uint64_t)w * th) >> 32);
+    w = 14324383u + (uint32_t)(((uint64_t)w * th) >> 32);
+    w = 185991442u + (uint32_t)(((uint64_t)w * th) >> 32);
+    w = 2146631446u + (uint32_t)(((uint64_t)w * th) >> 32);
+    uint64_t v = 0xa184897c363c4ull + sf_mulhi(t, (uint64_t)w << 17);
+    v = 0x5761ff9e299cc4ull + sf_mulhi(t, v);
+    v = 0x276556df749cee5ull + sf_mulhi(t, v);
+    v = 0xe35846b82505fc6ull + sf_mulhi(t, v);
+    v = 0x3d7f7bff058b1d51ull + sf_mulhi(t, v);
+    v = 0xb17217f7d1cf79acull + sf_mulhi(t, v);
+    v = (1ull << 63) + (sf_mulhi(t, v) >> 1);  // 2^t, Q1.63
+    const uint64_t k01 = (i & 1u) ? 0x9837f0518db8a96full : 0x8000000000000000ull;
+    const uint64_t k23 = (i & 1u) ? 0xd744fccad69d6af4ull : 0xb504f333f9de6484ull;
+    return Sf{sf_mulhi(v, (i & 2u) ? k23 : k01) << 1, n - 63};
+}
+
+}  // namespace vamp
