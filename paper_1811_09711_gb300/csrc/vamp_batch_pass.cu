@@ -12,8 +12,8 @@
 //
 // The item code is compiled for four dimension classes (d in 1..4, 5..8,
 // 9..12, 13..16): each unrolls its row loops to the class's largest d with
-// no test on the rows every member has, and the classes of small d process
-// two calls per thread.
+// no test on the rows every member has, and in FP32 the classes of small d
+// process two calls per thread.
 #include "vamp_pass.cuh"
 
 namespace vamp {
@@ -64,6 +64,8 @@ __device__ __forceinline__ bool run_item(const MultiArgs& M, const Params& P, Sm
         const int64_t base = a + bt * B, end = min(b, base + B);
         Calls<T, CPT, SH::DM> C;
         phase_a<T, 0, CPT>(P, sh, M.iter[inst], base, end, c, C);
+        SoftCall<SH::DM> soft;
+        if constexpr (sizeof(T) == 8) soft_prepare(P, sh, C.p[0], C.Aexp[0], soft);
         for (int t = 0; t < ntiles; ++t) {
             const int bb = streaming ? (int)(u & 1) : t;
             if (streaming || bt == 0) {
@@ -73,7 +75,7 @@ __device__ __forceinline__ bool run_item(const MultiArgs& M, const Params& P, Sm
                     H.abort = 1;
                 }
             }
-            if (!H.abort) tile_compute<T, 0, CPT>(P, sh, buf0 + bb * tile_bytes, t, tile, c, C);
+            if (!H.abort) tile_compute<T, 0, CPT>(P, sh, buf0 + bb * tile_bytes, t, tile, c, C, &soft);
             __syncthreads();
             if (H.abort) {
                 // let this CTA's copies in flight land (bounded), then give up
@@ -113,6 +115,7 @@ __device__ __forceinline__ bool run_item(const MultiArgs& M, const Params& P, Sm
 template <typename T, int MINB, bool STRAT>
 __global__ void __launch_bounds__(PASS_THREADS, MINB) k_pass_multi(MultiArgs M)
 {
+    constexpr int kTwo = sizeof(T) == 4 ? 2 : 1;
     static_assert(sizeof(Params) <= PARAMS_SLOT, "Params does not fit its shared-memory slot");
     extern __shared__ __align__(128) unsigned char smem[];
     SmemHead& H = *reinterpret_cast<SmemHead*>(smem);
@@ -163,8 +166,8 @@ __global__ void __launch_bounds__(PASS_THREADS, MINB) k_pass_multi(MultiArgs M)
         // pseudo-stratified instances: the generic shape, which carries the
         // cell digits and cell sums (compiled only into the STRAT form)
         if (STRAT && Ps.stratified) ok = run_item<T, 1, Shape<T, 0, 0>>(M, Ps, H, buf0, inst, c, kth, pp, bad);
-        else if (d <= 4) ok = run_item<T, 2, Shape<T, 0, 0, 4, 1>>(M, Ps, H, buf0, inst, c, kth, pp, bad);
-        else if (d <= 8) ok = run_item<T, 2, Shape<T, 0, 0, 8, 5>>(M, Ps, H, buf0, inst, c, kth, pp, bad);
+        else if (d <= 4) ok = run_item<T, kTwo, Shape<T, 0, 0, 4, 1>>(M, Ps, H, buf0, inst, c, kth, pp, bad);
+        else if (d <= 8) ok = run_item<T, kTwo, Shape<T, 0, 0, 8, 5>>(M, Ps, H, buf0, inst, c, kth, pp, bad);
         else if (d <= 12) ok = run_item<T, 1, Shape<T, 0, 0, 12, 9>>(M, Ps, H, buf0, inst, c, kth, pp, bad);
         else ok = run_item<T, 1, Shape<T, 0, 0, 16, 13>>(M, Ps, H, buf0, inst, c, kth, pp, bad);
         if (!ok) return;

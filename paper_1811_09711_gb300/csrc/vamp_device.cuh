@@ -16,15 +16,18 @@
 // the most bins any cell overlaps), so a lookup starts next to its answer.
 // Density entry n repeats entry n-1, so that a probe of edge ξ_n = 1 by a
 // point at (or rounded past) 1 needs no bounds check: it lands on entry n
-// with the last bin's density.  In the FP64 blocks the rows of mapped
-// coordinates hold the images φ_c(ξ_j) of the edges (and their cell table
-// is over p): the maps are increasing, so the bin of φ_c^{-1}(p) is the bin
-// whose image holds p, found with no inverse map.
+// with the last bin's density.  In the FP64 blocks the densities are packed
+// numbers (vamp_soft64.cuh), and the rows of mapped coordinates hold the
+// images φ_c(ξ_j) of the edges: the maps are increasing, so the bin of
+// φ_c^{-1}(p) is the bin whose image holds p, decided with no inverse map; the
+// cell table of such a row is over x, entered with an FP32 inverse map.
 #pragma once
 
 #include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
+
+#include "vamp_soft64.cuh"
 
 namespace vamp {
 
@@ -70,6 +73,24 @@ struct ChanHdr {
     uint32_t pad[(16 - (sizeof(T) + 4) % 16) % 16 / 4];
     T sp[MAXMAP][SP_N];  // per slot: m, Γ, A, Γ², 1/Γ, Γ/A, 1/A, atan(m/Γ), δ, 1/powN
 };
+// FP64: the mapped coordinates as a list, and what does not depend on the
+// call folded into two constants.
+template <>
+struct alignas(16) ChanHdr<double> {
+    uint32_t mask;       // bit k: coordinate k is mapped
+    uint32_t kinds;      // byte s: map kind of slot s
+    uint64_t slotpack;   // 4 bits per coordinate: its slot
+    double wz;           // matching peak: weight x Z^-(d - nmap)
+    uint32_t slow;       // bit k: some cell of (unmapped) row k overlaps more than two bins
+    uint32_t mmask;      // bit k: coordinate k has a Breit-Wigner or power-law map
+    double gN;           // Π_BW Γ/A x 0.2^(number of power-law slots): times α the constant of the term of g(p)
+    double fN;           // wz Π_BW Γ/A Π_POW 1/powN: the constant of the matching peak
+    uint32_t nslot;      // Breit-Wigner and power-law slots
+    uint8_t sk[MAXMAP];  // their coordinate | kind << 4
+    double c0[MAXMAP], c1[MAXMAP];    // Breit-Wigner: m, Γ²; power law: δ
+    float pinvG[MAXMAP], pt0[MAXMAP], pscale[MAXMAP];  // FP32 inverse map to cells: (atan(dp/Γ) + t0) scale; x scale
+    double sp[MAXMAP][SP_N];  // per slot: m, Γ, A, Γ², 1/Γ, Γ/A, 1/A, atan(m/Γ), δ, 1/powN
+};
 static_assert(sizeof(ChanHdr<float>) % 16 == 0 && sizeof(ChanHdr<double>) % 16 == 0, "header not 16-byte sized");
 
 // Byte layout of one channel's lookup block for element type T.
@@ -109,6 +130,8 @@ struct Scalars {
 // All pointers and sizes a kernel needs (passed by value).
 struct Params {
     int d, K, n, P;
+    uint32_t map_any, pow_any;  // bit k: some channel has a Breit-Wigner or power-law map (a power-law map) on k
+    int gauss_sum;         // the Gaussian factor of one coordinate can leave the packed range: exponents are summed
     int matching;          // peaks are the channels' maps (integrand fused into the channel loop)
     uint32_t key0, key1, request;
     int64_t n_min;
@@ -128,6 +151,7 @@ struct Params {
     double* edges64;   // [K][d][n+1] FP64 master grid
     double* alpha;     // [K]
     float* alpha32;    // [K]
+    double* alphaN;    // [K] α times the header's gN (kept with alpha32)
     double* shift;     // [K]
     double* Acum;      // [K] cumulative α for generation
     int64_t* Nc;       // [K]
@@ -475,7 +499,10 @@ __device__ __forceinline__ void forward_call(const Params& P, const SH& sh, int 
                              : reinterpret_cast<const T*>(row);
             x[k] = Prec<T>::lerp(__ldg(e + j), __ldg(e + j + 1), fr);
             jf[k] = j;
-            g *= __ldg(reinterpret_cast<const T*>(row + sh.dens_off()) + j);
+            if constexpr (sizeof(T) == 8)
+                g *= sf_unpack_double(__ldg(reinterpret_cast<const unsigned long long*>(row + sh.dens_off()) + j));
+            else
+                g *= __ldg(reinterpret_cast<const T*>(row + sh.dens_off()) + j);
         } else {
             x[k] = T(0);
             jf[k] = 0;
@@ -528,27 +555,17 @@ __device__ __forceinline__ void forward_call(const Params& P, const SH& sh, int 
 // bins, so one edge probe settles each bin and the unrolled row loop has no
 // branch other than the mapped-coordinate test; otherwise rows are tested
 // one by one and only the spanning ones search.
-// pw (FP64 pass kernel, else null): this thread's 0.2 p_k^(-4/5) per call q
-// and coordinate k at pw[(q DM + k) PASS_THREADS], computed once per call,
-// the power-law Jacobian of every channel that maps k.
+// (FP32; the FP64 form is soft_channel below.)
 template <typename T, int CPT, bool REC, bool FAST, class SH>
 __device__ __forceinline__ void channel_rows(const Params& P, const SH& sh, const unsigned char* blk, bool with_f,
                                              const T (&p)[CPT][SH::DM], T (&J)[CPT], T (&F)[CPT], T (&gp)[CPT],
-                                             T (&as)[CPT], int* bins, const T* pw)
+                                             T (&as)[CPT], int* bins)
 {
     const int d = sh.d();
     const ChanHdr<T>& h = *reinterpret_cast<const ChanHdr<T>*>(blk);
     const uint32_t mask = h.mask, kinds = h.kinds, slow = h.slow;
     const uint64_t slotpack = h.slotpack;
     const T gc = Prec<T>::gcen(P), k2 = Prec<T>::gk2(P);
-    // FP64: the Breit-Wigner Jacobians Γ/(A((p-m)² + Γ²)) of the channel as
-    // one quotient of the products of numerators and denominators (one FP64
-    // division per channel instead of one per mapped coordinate; each
-    // denominator is at least Γ², so the product of four stays normal)
-    T bw_num = T(1), bw_den[CPT];
-    bool any_bw = false;
-#pragma unroll
-    for (int q = 0; q < CPT; ++q) bw_den[q] = T(1);
 #pragma unroll
     for (int k = 0; k < SH::DM; ++k) {
         if (sh.has(k)) {
@@ -565,43 +582,21 @@ __device__ __forceinline__ void channel_rows(const Params& P, const SH& sh, cons
 #pragma unroll
                     for (int q = 0; q < CPT; ++q) {
                         const T dp = p[q][k] - mass;
-                        if constexpr (sizeof(T) == 8) {
-                            // FP64 rows of mapped coordinates hold the images of
-                            // the edges: the lookup compares p itself
-                            bw_den[q] *= dp * dp + G2;
-                        } else {
-                            const T jfac = Prec<T>::div(GinvA, dp * dp + G2);
-                            J[q] *= jfac;
-                            F[q] *= jfac;
-                            xk[q] = (Prec<T>::atan_(dp * invG) + t0) * invA;
-                        }
+                        const T jfac = Prec<T>::div(GinvA, dp * dp + G2);
+                        J[q] *= jfac;
+                        F[q] *= jfac;
+                        xk[q] = (Prec<T>::atan_(dp * invG) + t0) * invA;
                         const T u = p[q][k] - gc;
                         as[q] += u * u * k2;
-                    }
-                    if constexpr (sizeof(T) == 8) {
-                        bw_num *= GinvA;
-                        any_bw = true;
                     }
                 } else if (kind == MAP_POW) {
                     const T del = sp[SP_DEL], ipn = sp[SP_INVPOWN];
 #pragma unroll
                     for (int q = 0; q < CPT; ++q) {
-                        if constexpr (sizeof(T) == 8) {
-                            // 1/φ' = 1/(5 x^4) = y^4 / 5 with x = p^0.2 and
-                            // y = p^(-1/5): no division, no pow (the lookup
-                            // compares p with the edge images)
-                            if (pw) {
-                                J[q] *= pw[(q * SH::DM + k) * PASS_THREADS_DEV];
-                            } else {
-                                const T y = Prec<T>::rinv5(p[q][k]), y2 = y * y, y4 = y2 * y2;
-                                J[q] *= T(0.2) * y4;
-                            }
-                        } else {
-                            const T xx = Prec<T>::pow02(p[q][k]);
-                            const T x2 = xx * xx;
-                            J[q] *= Prec<T>::div(T(1), T(5) * (x2 * x2));
-                            xk[q] = xx;
-                        }
+                        const T xx = Prec<T>::pow02(p[q][k]);
+                        const T x2 = xx * xx;
+                        J[q] *= Prec<T>::div(T(1), T(5) * (x2 * x2));
+                        xk[q] = xx;
                         if (with_f) F[q] *= Prec<T>::powm08(p[q][k] + del) * ipn;
                         const T u = p[q][k] - gc;
                         as[q] += u * u * k2;
@@ -637,36 +632,178 @@ __device__ __forceinline__ void channel_rows(const Params& P, const SH& sh, cons
             }
         }
     }
-    if constexpr (sizeof(T) == 8) {
-        if (any_bw) {
-#pragma unroll
-            for (int q = 0; q < CPT; ++q) {
-                const T jb = Prec<T>::div(bw_num, bw_den[q]);
-                J[q] *= jb;
-                F[q] *= jb;
-            }
-        }
-    }
 }
 
 template <typename T, int CPT, bool REC, class SH>
 __device__ __forceinline__ void channel_body(const Params& P, const SH& sh, const unsigned char* blk, T alpha_c,
                                              bool lookups, bool with_f, const T (&p)[CPT][SH::DM],
                                              const T (&A)[CPT], const bool (&skip)[CPT], T (&g)[CPT],
-                                             T (&f)[CPT], int* bins, const T* pw = nullptr)
+                                             T (&f)[CPT], int* bins)
 {
     const ChanHdr<T>& h = *reinterpret_cast<const ChanHdr<T>*>(blk);
     T J[CPT], F[CPT], gp[CPT], as[CPT];
 #pragma unroll
     for (int q = 0; q < CPT; ++q) { J[q] = T(1); F[q] = T(1); gp[q] = T(1); as[q] = T(0); }
-    if (h.slow == 0u) channel_rows<T, CPT, REC, true>(P, sh, blk, with_f, p, J, F, gp, as, bins, pw);
-    else channel_rows<T, CPT, REC, false>(P, sh, blk, with_f, p, J, F, gp, as, bins, pw);
+    if (h.slow == 0u) channel_rows<T, CPT, REC, true>(P, sh, blk, with_f, p, J, F, gp, as, bins);
+    else channel_rows<T, CPT, REC, false>(P, sh, blk, with_f, p, J, F, gp, as, bins);
     const T wz = h.wz;
 #pragma unroll
     for (int q = 0; q < CPT; ++q) {
         if (lookups && !skip[q]) g[q] += alpha_c * gp[q] * J[q];
         if (with_f) f[q] += wz * Prec<T>::exp2_(as[q] - A[q]) * F[q];
     }
+}
+
+// ---------------------------------------------------------------------------
+// The FP64 form of the channel loop, on the integer pipe (vamp_soft64.cuh).
+// Same terms as channel_body: g += α_c g_c(φ_c^{-1}(p)) / φ'_c, f += the
+// matching peak.  What bounded it before: the FP64 pipe, 76 % busy with about
+// 5 200 operations a call on the collider (d = 14, K = 64), 134 ms per 1e7
+// calls.  Here the FP64 pipe keeps, per channel, p - m and (p - m)² + Γ² of
+// each Breit-Wigner slot, p + δ of each power-law slot and the two sums.
+// ---------------------------------------------------------------------------
+// Per call, for all channels: the cell of p_k in an unmapped row's table (the
+// same for every channel), and for coordinates that some channel maps the
+// Gaussian factor 2^(a_k) that its peak must not have (its exponent a_k, where
+// P.gauss_sum is set) and p_k^(-4/5).  The arrays that the slots index by coordinate live in local memory (coalesced
+// there, and read at most 4 times a channel).
+template <int DM>
+struct SoftCall {
+    int q[DM];
+    double p[DM];
+    uint64_t E[DM], W[DM];
+    Sf e0;     // 2^-(Σ a_k), the Gaussian factors of all coordinates (1 where P.gauss_sum)
+    double A;  // Σ a_k
+};
+
+template <class SH>
+__device__ __forceinline__ void soft_prepare(const Params& P, const SH& sh, const double (&p)[SH::DM], double A,
+                                             SoftCall<SH::DM>& S)
+{
+#pragma unroll
+    for (int k = 0; k < SH::DM; ++k) {
+        if (sh.has(k)) {
+            S.q[k] = Prec<double>::cell(p[k], sh.lshift());
+            S.p[k] = p[k];
+        }
+    }
+    for (uint32_t m = P.map_any; m; m &= m - 1u) {
+        const int k = __ffs(m) - 1;
+        const double pk = S.p[k];
+        if (P.matching) {
+            const double u = pk - P.gcen;
+            const double a = u * u * P.gk2;
+            S.E[k] = P.gauss_sum ? sf_bits(a) : sf_pack(sf_exp2(a));
+        }
+        if ((P.pow_any >> k) & 1u) S.W[k] = sf_pack(sf_powm08(pk));
+    }
+    S.A = A;
+    S.e0 = P.matching && !P.gauss_sum ? sf_exp2(-A) : Sf{1ull << 63, -63};
+}
+
+// One packed factor onto acc; the exponents' biases are added by the caller.
+__device__ __forceinline__ void soft_factor(uint64_t& acc, int& ae, uint64_t w)
+{
+    acc = sf_mulhi(acc, w & ~2047ull);
+    ae += (int)((uint32_t)w & 2047u);
+}
+
+// Channel c' (block in shared or global memory) against one call: its term of
+// g(p) without the constant α gN, and of f without fN.  bins (REC): the bin of
+// every row.
+template <bool REC, class SH>
+__device__ __forceinline__ void soft_channel(const Params& P, const SH& sh, const unsigned char* blk, bool lookups,
+                                             const double (&p)[SH::DM], const SoftCall<SH::DM>& S, double& gt,
+                                             double& ft, int* bins)
+{
+    const bool with_f = P.matching != 0, gauss_sum = P.gauss_sum != 0;
+    const ChanHdr<double>& h = *reinterpret_cast<const ChanHdr<double>*>(blk);
+    const uint32_t mmask = h.mmask;
+    const int n = sh.n();
+    uint64_t acc = 1ull << 63;
+    int ae = 0, rows = 0;  // acc 2^(ae - 1022 rows - 63)
+    if (lookups) {
+        if (h.slow == 0u) {
+#pragma unroll
+            for (int k = 0; k < SH::DM; ++k) {
+                if (sh.has(k) && !((mmask >> k) & 1u)) {
+                    const unsigned char* row = sh.row(blk, k);
+                    const double* e = reinterpret_cast<const double*>(row);
+                    int j = row[sh.tab_off() + S.q[k]];
+                    j += Prec<double>::le(e[j + 1], p[k]) ? 1 : 0;
+                    if (REC) bins[k] = min(j, n - 1);
+                    soft_factor(acc, ae, reinterpret_cast<const uint64_t*>(row + sh.dens_off())[j]);
+                }
+                if (k % 4 == 3) {  // four factors lose at most four leading bits
+                    const int z = sf_clz(acc);
+                    acc <<= z;
+                    ae -= z;
+                }
+            }
+            rows = sh.d() - __popc(mmask);
+        } else {
+            for (int k = 0; k < sh.d(); ++k) {
+                if ((mmask >> k) & 1u) continue;
+                const unsigned char* row = sh.row(blk, k);
+                const double* e = reinterpret_cast<const double*>(row);
+                const double pk = S.p[k];
+                int j = row[sh.tab_off() + Prec<double>::cell(pk, sh.lshift())];
+                for (int s = 128; s > 0; s >>= 1)  // largest j with e[j] <= p
+                    if (j + s < n && Prec<double>::le(e[j + s], pk)) j += s;
+                if (REC) bins[k] = j;
+                soft_factor(acc, ae, reinterpret_cast<const uint64_t*>(row + sh.dens_off())[j]);
+                const int z = sf_clz(acc);
+                acc <<= z;
+                ae -= z;
+                ++rows;
+            }
+        }
+    }
+    const Sf one{1ull << 63, -63};
+    Sf den = one, G = one, F = S.e0;
+    double as = 0.0;
+    bool any_bw = false;
+#pragma unroll 1
+    for (uint32_t s = 0; s < h.nslot; ++s) {
+        const int k = h.sk[s] & 15;
+        const double pk = S.p[k];
+        float xc;  // cell of the FP32 inverse map, a fraction of a cell low
+        if ((h.sk[s] >> 4) == MAP_BW) {
+            const double dp = pk - h.c0[s];
+            den = sf_norm(sf_mul(den, sf_from_double(dp * dp + h.c1[s])));
+            any_bw = true;
+            xc = (atanf(sf_to_float(dp) * h.pinvG[s]) + h.pt0[s]) * h.pscale[s];
+        } else {
+            if (with_f) F = sf_norm(sf_mul(F, sf_powm08(pk + h.c0[s])));
+            G = sf_norm(sf_mul(G, sf_unpack(S.W[k])));
+            const uint64_t b = sf_bits(pk);
+            const float lg = sf_lg2f((float)(((uint32_t)(b >> 29) & 0x7fffffu) | 0x800000u)) + (float)((int)((int64_t)b >> 52) - 1046);
+            // (p < 0, by rounding at a map's lower end, gives cell 0)
+            xc = sf_ex2f(0.2f * lg) * h.pscale[s];
+        }
+        if (with_f) {
+            if (gauss_sum) as += sf_from_bits(S.E[k]);
+            else F = sf_norm(sf_mul(F, sf_unpack(S.E[k])));
+        }
+        if (lookups) {
+            const unsigned char* row = sh.row(blk, k);
+            const double* e = reinterpret_cast<const double*>(row);
+            const int L = 1 << sh.lshift();
+            int j = row[sh.tab_off() + min(max((int)(xc - 0.02f), 0), L)];
+            while (j < n - 1 && Prec<double>::le(e[j + 1], pk)) ++j;
+            if (REC) bins[k] = j;
+            soft_factor(acc, ae, reinterpret_cast<const uint64_t*>(row + sh.dens_off())[j]);
+            const int z = sf_clz(acc);
+            acc <<= z;
+            ae -= z;
+            ++rows;
+        }
+    }
+    if (with_f && gauss_sum) F = sf_norm(sf_mul(F, sf_exp2(as - S.A)));
+    const Sf y = any_bw ? sf_rcp(den) : one;
+    const Sf a{acc, ae - 1022 * rows - 63};
+    gt = lookups ? sf_to_double(sf_norm(sf_mul(sf_mul(a, G), y))) : 0.0;
+    ft = with_f ? sf_to_double(sf_norm(sf_mul(F, y))) : 0.0;
 }
 
 // Integrand of a non-matching problem: loop over its own peaks.

@@ -92,7 +92,7 @@ bool build_setup(const vamp_config* cfg, Params& P, Setup& S, std::string& why);
 
 // Device-side placement of the per-problem arrays inside one buffer.
 struct Arena {
-    size_t edges64, lk64, lk32, alpha, alpha32, shift, acum, nc, pc, D, csum, ic, vc, wc, pk64, pk32, sc;
+    size_t edges64, lk64, lk32, alpha, alpha32, alphan, shift, acum, nc, pc, D, csum, ic, vc, wc, pk64, pk32, sc;
     size_t nr, spc, coff, qc;
     size_t eqoff, eqent;   // 0 bytes without equivalences
     size_t bytes;

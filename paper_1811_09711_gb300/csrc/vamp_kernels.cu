@@ -220,9 +220,8 @@ __device__ __forceinline__ void derive_row_t(const Params& P, const BlkLayout& L
     unsigned char* tb = r + (L.Es + L.Dn) * sizeof(T);
     // FP64 rows of mapped coordinates hold the images φ_c(ξ_j) of the edges
     // (clamped at 0, the forward map's formula): a bin of x = φ_c^{-1}(p) is
-    // the bin whose image holds p, so the FP64 lookups compare p itself and
-    // need no inverse map; the forward map reads the edges from the master
-    // grid
+    // the bin whose image holds p, so the FP64 lookups compare p itself; the
+    // forward map reads the edges from the master grid
     int kind = MAP_ID;
     const double* sp = nullptr;
     if (sizeof(T) == 8) {
@@ -244,17 +243,21 @@ __device__ __forceinline__ void derive_row_t(const Params& P, const BlkLayout& L
         }
         e[j] = (T)(v > 0.0 ? v : 0.0);
         const int jb = j < n ? j : n - 1;  // entry n repeats bin n-1
-        dnr[j] = (T)(1.0 / ((double)n * (e64[jb + 1] - e64[jb])));
+        const double dens = 1.0 / ((double)n * (e64[jb + 1] - e64[jb]));
+        if constexpr (sizeof(T) == 8) reinterpret_cast<uint64_t*>(dnr)[j] = sf_pack_double(dens);
+        else dnr[j] = (T)dens;
     }
     __syncwarp();
-    // tb[q] = largest j in [0, n-1] with e[j] <= q/L, for q = 0..L
+    // tb[q] = largest j in [0, n-1] with e[j] <= q/L, for q = 0..L (over x
+    // in the FP64 rows of mapped coordinates)
     const int Lc = 1 << L.lshift;
+    const bool over_x = sizeof(T) == 8 && kind != MAP_ID;
     for (int q = lane; q <= Lc; q += nl) {
         const T xq = (T)q / (T)Lc;
         int lo = 0, hi = n - 1;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
-            if (e[mid] <= xq) lo = mid; else hi = mid - 1;
+            if ((over_x ? (T)e64[mid] : e[mid]) <= xq) lo = mid; else hi = mid - 1;
         }
         tb[q] = (unsigned char)lo;
     }
@@ -267,9 +270,16 @@ __device__ __forceinline__ void derive_row_t(const Params& P, const BlkLayout& L
         tb[Lc + 1] = (unsigned char)min(span, 255);
         // this row's bit of the channel's slow-row mask (each row owns its bit)
         unsigned int* slow = reinterpret_cast<unsigned int*>(lk + (size_t)c * L.bytes + offsetof(ChanHdr<T>, slow));
-        if (span > 1) atomicOr(slow, 1u << k);
+        if (span > 1 && !over_x) atomicOr(slow, 1u << k);
         else atomicAnd(slow, ~(1u << k));
     }
+}
+
+// The forms of α_c that the pass kernels read beside alpha[c].
+__device__ __forceinline__ void store_alpha(const Params& P, int c, double a)
+{
+    P.alpha32[c] = (float)a;
+    P.alphaN[c] = a * reinterpret_cast<const ChanHdr<double>*>(P.lk64 + (size_t)c * P.lay64.bytes)->gN;
 }
 
 __device__ __forceinline__ void derive_row(const Params& P, int row, int lane)
@@ -286,7 +296,7 @@ __global__ void k_derive(Params P)
     const int nw = gridDim.x * (blockDim.x >> 5);
     for (int row = w; row < rows; row += nw) derive_row(P, row, lane);
     if (blockIdx.x == 0)
-        for (int c = threadIdx.x; c < P.K; c += blockDim.x) P.alpha32[c] = (float)P.alpha[c];
+        for (int c = threadIdx.x; c < P.K; c += blockDim.x) store_alpha(P, c, P.alpha[c]);
 }
 
 // ---------------------------------------------------------------------------
@@ -439,7 +449,7 @@ __device__ void update_alpha_dev(const Params& P)
     const double tot = red[0];
     for (int c = threadIdx.x; c < K; c += blockDim.x) {
         if (tot > 0.0) P.alpha[c] = P.Acum[c] / tot;
-        P.alpha32[c] = (float)P.alpha[c];
+        store_alpha(P, c, P.alpha[c]);
     }
 }
 
@@ -550,7 +560,6 @@ __global__ void k_eval(Params P, EvalArgs A)
         c = choose_channel(P, unif64(xc));
     }
     T x[DMAX], p1[1][DMAX], g[1], f[1], Aq[1];
-    bool skip[1];
     int jf[DMAX];
     T owngJ;
     if (A.mode == 0 && P.stratified) {
@@ -568,12 +577,21 @@ __global__ void k_eval(Params P, EvalArgs A)
     g[0] = Prec<T>::alpha(P, c) * owngJ;
     f[0] = P.matching ? T(0) : integrand_peaks<T, DMAX>(P, d, p1[0], Aq[0]);
     int* bins = A.bins + (size_t)q * P.K * d;
+    SoftCall<DMAX> soft;
+    if constexpr (sizeof(T) == 8) soft_prepare(P, sh, p1[0], Aq[0], soft);
     for (int c2 = 0; c2 < P.K; ++c2) {
         const T a = Prec<T>::alpha(P, c2);
         const bool lookups = a != T(0) && c2 != c;
-        skip[0] = false;
         const unsigned char* blk = Prec<T>::lk(P) + (size_t)c2 * sh.bytes();
-        channel_body<T, 1, true>(P, sh, blk, a, lookups, P.matching != 0, p1, Aq, skip, g, f, bins + c2 * d);
+        if constexpr (sizeof(T) == 8) {
+            double gt, ft;
+            soft_channel<true>(P, sh, blk, lookups, p1[0], soft, gt, ft, bins + c2 * d);
+            if (lookups) g[0] += P.alphaN[c2] * gt;
+            if (P.matching) f[0] += reinterpret_cast<const ChanHdr<double>*>(blk)->fN * ft;
+        } else {
+            const bool skip[1] = {false};
+            channel_body<T, 1, true>(P, sh, blk, a, lookups, P.matching != 0, p1, Aq, skip, g, f, bins + c2 * d);
+        }
         if (a == T(0))
             for (int k = 0; k < d; ++k) bins[c2 * d + k] = -1;
         else if (c2 == c)

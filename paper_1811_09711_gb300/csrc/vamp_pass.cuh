@@ -147,19 +147,28 @@ __device__ __forceinline__ void phase_a(const Params& P, const SH& sh, uint32_t 
 // Phase B for one staged tile: channels t*tile .. of the tile buffer tb.
 template <typename T, int MODE, int CPT, class SH>
 __device__ __forceinline__ void tile_compute(const Params& P, const SH& sh, const unsigned char* tb, int t, int tile,
-                                             int cseg, Calls<T, CPT, SH::DM>& C, const T* pw = nullptr)
+                                             int cseg, Calls<T, CPT, SH::DM>& C, const SoftCall<SH::DM>* soft)
 {
     const int S = sh.bytes();
     const int cnt = min(tile, P.K - t * tile);
-    bool skip[CPT];
     for (int cl = 0; cl < cnt; ++cl) {
         const int c2 = t * tile + cl;
-        const T a = Prec<T>::alpha(P, c2);
-        const bool lookups = (a != T(0)) && !(MODE == 0 && c2 == cseg);
+        const unsigned char* blk = tb + (size_t)cl * S;
+        if constexpr (sizeof(T) == 8) {
+            const double a = __ldg(P.alphaN + c2);
+            const bool lookups = (a != 0.0) && !(MODE == 0 && c2 == cseg);
+            double gt, ft;
+            soft_channel<false>(P, sh, blk, lookups, C.p[0], *soft, gt, ft, nullptr);
+            if (lookups && !(MODE == 1 && C.cq[0] == c2)) C.g[0] += a * gt;
+            if (P.matching) C.f[0] += reinterpret_cast<const ChanHdr<double>*>(blk)->fN * ft;
+        } else {
+            bool skip[CPT];
+            const T a = Prec<T>::alpha(P, c2);
+            const bool lookups = (a != T(0)) && !(MODE == 0 && c2 == cseg);
 #pragma unroll
-        for (int q = 0; q < CPT; ++q) skip[q] = (MODE == 1) && (C.cq[q] == c2);
-        channel_body<T, CPT, false>(P, sh, tb + (size_t)cl * S, a, lookups, P.matching != 0, C.p, C.Aexp, skip,
-                                    C.g, C.f, nullptr, pw);
+            for (int q = 0; q < CPT; ++q) skip[q] = (MODE == 1) && (C.cq[q] == c2);
+            channel_body<T, CPT, false>(P, sh, blk, a, lookups, P.matching != 0, C.p, C.Aexp, skip, C.g, C.f, nullptr);
+        }
     }
 }
 
@@ -329,20 +338,7 @@ __global__ void __launch_bounds__(PASS_THREADS, MINB) k_pass(Params P, PassArgs 
     const int tid = threadIdx.x;
     constexpr int B = PASS_THREADS * CPT;
     const unsigned char* lk = Prec<T>::lk(P);
-    // FP64: the power-law Jacobian 0.2 p_k^(-4/5) of each coordinate of this
-    // thread's call, computed once per call instead of once per channel that
-    // maps k (after the tiles and the d-values; DMAX x PASS_THREADS doubles
-    // are reserved by pass_smem)
-    constexpr bool kPW = sizeof(T) == 8 && CPT == 1;
-    T* pwS = nullptr;
-    if constexpr (kPW) {
-        // used only where the launch reserved the space (see pass_smem)
-        unsigned dsm = 0;
-        asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dsm));
-        const size_t off = SMEM_HEAD + tiles_bytes + (MODE == 0 ? (size_t)(dn << A.dshift) * 8 : 0);
-        if ((size_t)dsm >= off + (size_t)DM * PASS_THREADS * sizeof(T))
-            pwS = reinterpret_cast<T*>(smem + off);
-    }
+    SoftCall<DM> soft;  // FP64: what the channel loop needs of the call
 
     // ---- work of this CTA ---------------------------------------------------
     int64_t r0 = 0, r1 = 0;
@@ -422,16 +418,9 @@ __global__ void __launch_bounds__(PASS_THREADS, MINB) k_pass(Params P, PassArgs 
         Calls<T, CPT, DM> C;
         const bool live = MODE == 1 || base + warp_first<CPT>() < end;  // some call of this warp
         if (live) phase_a<T, MODE, CPT>(P, sh, A.field, base, end, cseg, C);
-        if constexpr (kPW) {
-            if (live && pwS) {
-#pragma unroll
-                for (int k = 0; k < DM; ++k) {
-                    if (sh.has(k)) {
-                        const T y = Prec<T>::rinv5(C.p[0][k]), y2 = y * y;
-                        pwS[k * PASS_THREADS + tid] = T(0.2) * (y2 * y2);
-                    }
-                }
-            }
+        if constexpr (sizeof(T) == 8) {
+            static_assert(CPT == 1, "the FP64 channel loop takes one call per thread");
+            if (live) soft_prepare(P, sh, C.p[0], C.Aexp[0], soft);
         }
 
         // ---- phase B: every channel's term of g(p) (and the matching peaks) --
@@ -446,7 +435,7 @@ __global__ void __launch_bounds__(PASS_THREADS, MINB) k_pass(Params P, PassArgs 
                 }
             }
             if (live && !H.abort)
-                tile_compute<T, MODE, CPT>(P, sh, buf0 + b * tile_bytes, t, A.tile, cseg, C, pwS ? pwS + tid : nullptr);
+                tile_compute<T, MODE, CPT>(P, sh, buf0 + b * tile_bytes, t, A.tile, cseg, C, &soft);
             __syncthreads();
             if (H.abort) goto drain;
             if (streaming && tid == 0 && issued < total_uses) {

@@ -85,7 +85,7 @@ MapRec<T> make_rec(const vamp_map_desc& r, double weight, double zinv, int d)
 }
 
 template <typename T>
-void make_hdr(const vamp_map_desc& r, double weight, double zinv, int d, unsigned char* out)
+void make_hdr(const vamp_map_desc& r, double weight, double zinv, int d, int lshift, unsigned char* out)
 {
     ChanHdr<T> h;
     std::memset(&h, 0, sizeof h);
@@ -109,6 +109,40 @@ void make_hdr(const vamp_map_desc& r, double weight, double zinv, int d, unsigne
         } else if (r.kind[s] == VAMP_MAP_POW) {
             sp[SP_DEL] = (T)r.b[s];
             sp[SP_INVPOWN] = (T)pow_invN(r.b[s]);
+        }
+    }
+    if constexpr (sizeof(T) == 8) {
+        // the slots with a factor, and the constants of the channel's terms
+        // (SoftCall); a map whose constants are not finite makes them so too,
+        // and with them the weights, which are then reported
+        h.gN = 1.0;
+        h.fN = h.wz;
+        for (int s = 0; s < r.n_mapped; ++s) {
+            const int kind = r.kind[s], q = (int)h.nslot;
+            if (kind != MAP_BW && kind != MAP_POW) continue;
+            h.mmask |= 1u << r.coord[s];
+            h.sk[q] = (uint8_t)(r.coord[s] | kind << 4);
+            // cells of the row's table per unit of the FP32 inverse map, whose
+            // error (about 4e-7 / A) must stay below the 0.02 cells that the
+            // lookup allows it; 0: the search starts at the first bin
+            const double cells = (double)(1 << lshift);
+            if (kind == MAP_BW) {
+                const double A = h.sp[s][SP_A];
+                h.c0[q] = h.sp[s][SP_M];
+                h.c1[q] = h.sp[s][SP_G2];
+                h.gN *= h.sp[s][SP_GINVA];
+                h.fN *= h.sp[s][SP_GINVA];
+                if (!(h.sp[s][SP_G2] >= 2.3e-308)) h.gN = h.fN = NAN;  // Γ² vanishes
+                h.pinvG[q] = (float)h.sp[s][SP_INVG];
+                h.pt0[q] = (float)h.sp[s][SP_T0];
+                h.pscale[q] = A > 0.3 ? (float)(cells / A) : 0.f;
+            } else {
+                h.c0[q] = h.sp[s][SP_DEL];
+                h.gN *= 0.2;
+                h.fN *= h.sp[s][SP_INVPOWN];
+                h.pscale[q] = (float)cells;
+            }
+            ++h.nslot;
         }
     }
     std::memcpy(out, &h, sizeof h);
@@ -185,6 +219,7 @@ bool build_setup(const vamp_config* cfg, Params& pr, Setup& S, std::string& why)
     // gk2 = log2(e) / (2σ²); σ = 0 switches it off (factor 1)
     S.zinv = 1.0;
     pr.gcen = 0.0; pr.gk2 = 0.0; pr.gcen_f = 0.f; pr.gk2_f = 0.f;
+    pr.gauss_sum = 0;
     if (cfg->gauss_sigma > 0.0) {
         const double s = cfg->gauss_sigma, cc = cfg->gauss_centre;
         double Z;
@@ -193,12 +228,22 @@ bool build_setup(const vamp_config* cfg, Params& pr, Setup& S, std::string& why)
         S.zinv = 1.0 / Z;
         pr.gcen = cc;
         pr.gk2 = M_LOG2E / (2.0 * s * s);
+        // a coordinate's exponent reaches this; packed numbers hold up to 2^960
+        const double amax = std::max(cc * cc, (1.0 - cc) * (1.0 - cc)) * pr.gk2;
+        pr.gauss_sum = amax > 900.0;
         pr.gcen_f = (float)cc;
         pr.gk2_f = (float)pr.gk2;
     }
     pr.matching = P == K;
     for (int q = 0; pr.matching && q < K; ++q)
         if (!same_maps(cfg->channels[q], cfg->peaks[q])) pr.matching = 0;
+    pr.map_any = pr.pow_any = 0;
+    for (int q = 0; q < K; ++q)
+        for (int t = 0; t < cfg->channels[q].n_mapped; ++t) {
+            const int kind = cfg->channels[q].kind[t];
+            if (kind != VAMP_MAP_ID) pr.map_any |= 1u << cfg->channels[q].coord[t];
+            if (kind == VAMP_MAP_POW) pr.pow_any |= 1u << cfg->channels[q].coord[t];
+        }
     pr.lay64 = make_layout_c<double>(d, n);
     pr.lay32 = make_layout_c<float>(d, n);
 
@@ -207,8 +252,8 @@ bool build_setup(const vamp_config* cfg, Params& pr, Setup& S, std::string& why)
     for (int q = 0; q < K; ++q) {
         // with matching peaks the channel header carries the peak weight too
         const double w = pr.matching ? cfg->peak_weight[q] : 0.0;
-        make_hdr<double>(cfg->channels[q], w, S.zinv, d, S.hdr64.data() + (size_t)q * pr.lay64.H);
-        make_hdr<float>(cfg->channels[q], w, S.zinv, d, S.hdr32.data() + (size_t)q * pr.lay32.H);
+        make_hdr<double>(cfg->channels[q], w, S.zinv, d, pr.lay64.lshift, S.hdr64.data() + (size_t)q * pr.lay64.H);
+        make_hdr<float>(cfg->channels[q], w, S.zinv, d, pr.lay32.lshift, S.hdr32.data() + (size_t)q * pr.lay32.H);
     }
     S.pk64.assign((size_t)P * sizeof(MapRec<double>), 0);
     S.pk32.assign((size_t)P * sizeof(MapRec<float>), 0);
@@ -232,6 +277,7 @@ Arena plan_arena(const Params& P)
     A.lk32 = take(K * P.lay32.bytes);
     A.alpha = take(K * 8);
     A.alpha32 = take(K * 4);
+    A.alphan = take(K * 8);
     A.shift = take(K * 8);
     A.acum = take(K * 8);
     A.nc = take(K * 8);
@@ -261,6 +307,7 @@ void bind_arena(Params& P, unsigned char* b, const Arena& A)
     P.lk32 = b + A.lk32;
     P.alpha = (double*)(b + A.alpha);
     P.alpha32 = (float*)(b + A.alpha32);
+    P.alphaN = (double*)(b + A.alphan);
     P.shift = (double*)(b + A.shift);
     P.Acum = (double*)(b + A.acum);
     P.Nc = (int64_t*)(b + A.nc);
@@ -332,16 +379,7 @@ TilePlan pass_smem(const Params& P, int fp32, int minb)
         cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) == cudaSuccess)
         budget = std::min(budget, (size_t)(per_sm / minb - reserved));
-    // FP64: each thread's power-law Jacobians of its call, one per coordinate,
-    // where they fit beside one tile in a block's largest shared memory (the
-    // kernel computes them per channel otherwise)
-    size_t pw = fp32 ? 0 : (size_t)DMAX * PASS_THREADS * 8;
-    int maxsm = 0;
-    if (pw && cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
-        SMEM_HEAD + 2 * S + (size_t)P.d * P.n * 8 + pw > (size_t)maxsm)
-        pw = 0;
-    return plan_tiles(S, P.K, P.d * P.n, SMEM_HEAD + pw, budget);
+    return plan_tiles(S, P.K, P.d * P.n, SMEM_HEAD, budget);
 }
 
 std::vector<const PassVariant*> pass_candidates(int fp32, int d, int n, int stratified, int K)

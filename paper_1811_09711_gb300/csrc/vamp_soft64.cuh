@@ -123,6 +123,22 @@ VAMP_HD uint64_t sf_pack(Sf a)
     return (r << 11) | (1ull << 63) | (uint32_t)x;
 }
 
+// x in FP32, truncated; 0 below the normal range.
+VAMP_HD float sf_to_float(double x)
+{
+    const uint64_t b = sf_bits(x);
+    const uint32_t hi = (uint32_t)(b >> 32), e = (hi >> 20) & 0x7ffu;
+    uint32_t r = (hi & 0x80000000u) | ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | ((uint32_t)b >> 29);
+    r = e < 897u ? 0u : (e > 1150u ? (hi & 0x80000000u) | 0x7f7fffffu : r);
+#ifdef __CUDA_ARCH__
+    return __uint_as_float(r);
+#else
+    float f;
+    std::memcpy(&f, &r, 4);
+    return f;
+#endif
+}
+
 VAMP_HD float sf_lg2f(float v)
 {
 #ifdef __CUDA_ARCH__
@@ -220,7 +236,7 @@ VAMP_HD Sf sf_powm08(double v)
     return sf_norm(Sf{z, -60 - 4 * a});
 }
 
-// 2^x of a finite double |x| < 2^20, normalised, to about 2^-57: the fraction's
+// 2^x of a finite double (|x| >= 2^20 as 2^±(2^20)), to about 2^-57, normalised: the fraction's
 // leading two bits pick 2^(i/4), the rest goes through the series of 2^t =
 // sum (t ln 2)^k / k! for t in [0, 1/4), whose terms from t^7 on (below 2^-30)
 // are summed in 32 bits.
@@ -232,9 +248,12 @@ VAMP_HD Sf sf_exp2(double x)
     // integer part and 64-bit fraction of |x|
     int n = 0;
     uint64_t f;
-    if (ex >= 0) {
+    if (ex >= 20) {
+        n = 1 << 20;
+        f = 0ull;
+    } else if (ex >= 0) {
         n = (int)(mant >> (63 - ex));
-        f = ex < 63 ? mant << (ex + 1) : 0ull;
+        f = mant << (ex + 1);
     } else {
         f = ex >= -64 ? mant >> (-1 - ex) : 0ull;
     }

@@ -95,3 +95,32 @@ BW, POW = P.MAP_BW, P.MAP_POW
 ])
 def test_d_value_copies_and_warp_cuts(V, O, d, n, K, calls):
     check_runs(V, O, problem(d, n, K, [[], [BW]]), 2, calls)
+
+
+@pytest.mark.parametrize("label,kw,iters,calls", [
+    ("all power, delta 0", dict(d=4, n=33, K=4, kinds=[[POW, POW, POW, POW]], deltas=(0.0, 0.0)), 2, 20_000),
+    ("four Breit-Wigners", dict(d=5, n=50, K=6, kinds=[[BW, BW, BW, BW], [BW]]), 2, 20_000),
+    ("mixed slots, 64 channels", dict(d=7, n=100, K=64, kinds=[[BW, POW, BW], [POW], [], [BW, POW, POW, BW]]), 2, 40_000),
+    ("peaks beside the channels", dict(d=6, n=31, K=9, kinds=[[BW, POW], [BW]], peaks_apart=True), 2, 20_000),
+    ("narrow", dict(d=3, n=64, K=5, kinds=[[BW, POW], [BW]], widths=(1e-7, 1e-6), deltas=(1e-9, 1e-8)), 1, 20_000),
+    ("no Gaussian", dict(d=3, n=20, K=3, kinds=[[BW], [POW]], sigma=0.0), 2, 20_000),
+    ("exponents of 100", dict(d=9, n=20, K=3, kinds=[[BW], [POW]], sigma=0.04), 1, 20_000),
+    ("exponents of 1800: summed", dict(d=4, n=20, K=3, kinds=[[BW], [POW]], sigma=0.01), 1, 20_000),
+    ("largest", dict(d=16, n=256, K=3, kinds=[[BW, POW, BW, POW]]), 1, 5_003),
+    ("one bin", dict(d=2, n=1, K=3, kinds=[[BW, POW], [POW]]), 1, 5_003),
+])
+def test_fp64_channel_products(V, O, label, kw, iters, calls):
+    """The FP64 channel loop multiplies 64-bit mantissas and finds the bins of
+    mapped coordinates from an FP32 inverse map: every pattern of slots, power
+    laws down to p = tiny, Gaussian exponents beyond a packed number's."""
+    check_runs(V, O, problem(**kw), iters, calls)
+
+
+def test_fp64_map_far_outside(V, O):
+    """Breit-Wigner maps whose mass lies far outside [0, 1] for their width
+    (A below 0.3): the FP32 inverse map is no guide and the search starts at bin 0."""
+    pr = problem(3, 40, 3, [[BW], []])
+    for ms in (pr.channels, pr.peaks):
+        ms.a[0, 0], ms.b[0, 0] = 1.8, 0.05
+        ms.a[2, 0], ms.b[2, 0] = -3.0, 0.5
+    check_runs(V, O, pr, 2, 20_000)
