@@ -86,6 +86,7 @@ struct alignas(16) ChanHdr<double> {
     double gN;           // Π_BW Γ/A x 0.2^(number of power-law slots): times α the constant of the term of g(p)
     double fN;           // wz Π_BW Γ/A Π_POW 1/powN: the constant of the matching peak
     uint32_t nslot;      // Breit-Wigner and power-law slots
+    uint32_t bw;         // some are Breit-Wigner
     uint8_t sk[MAXMAP];  // their coordinate | kind << 4
     double c0[MAXMAP], c1[MAXMAP];    // Breit-Wigner: m, Γ²; power law: δ
     float pinvG[MAXMAP], pt0[MAXMAP], pscale[MAXMAP];  // FP32 inverse map to cells: (atan(dp/Γ) + t0) scale; x scale
@@ -708,9 +709,36 @@ __device__ __forceinline__ void soft_factor(uint64_t& acc, int& ae, uint64_t w)
     ae += (int)((uint32_t)w & 2047u);
 }
 
+// Largest j' in [j, n] with e[j'] <= x, for e[j] <= x: three edges at a time,
+// since a search from the right cell seldom goes further.
+__device__ __forceinline__ int soft_search(const double* e, int j, int n, double x)
+{
+    for (;;) {
+        const int a = Prec<double>::le(e[min(j + 1, n)], x) ? 1 : 0, b = Prec<double>::le(e[min(j + 2, n)], x) ? 1 : 0,
+                  c = Prec<double>::le(e[min(j + 3, n)], x) ? 1 : 0;
+        j += a + b + c;
+        if (!c || j >= n) return min(j, n);
+    }
+}
+
+// atan t within 1.7e-6: the least-squares odd polynomial of degree 11 on
+// [0, 1], with atan t = pi/2 - atan(1/t) above.  A starting point of searches.
+__device__ __forceinline__ float atan_start(float t)
+{
+    const float a = fabsf(t), u = a > 1.f ? sf_rcpf(a) : a, v = u * u;
+    float y = fmaf(v, -0.011719031f, 0.052647073f);
+    y = fmaf(y, v, -0.116426215f);
+    y = fmaf(y, v, 0.19354026f);
+    y = fmaf(y, v, -0.3326228f);
+    y = fmaf(y, v, 0.99997723f) * u;
+    y = a > 1.f ? 1.57079633f - y : y;
+    return copysignf(y, t);
+}
+
 // Channel c' (block in shared or global memory) against one call: its term of
 // g(p) without the constant α gN, and of f without fN.  bins (REC): the bin of
-// every row.
+// every row.  At most eight factors follow one another without normalising
+// (each loses at most one of the 64 bits).
 template <bool REC, class SH>
 __device__ __forceinline__ void soft_channel(const Params& P, const SH& sh, const unsigned char* blk, bool lookups,
                                              const double (&p)[SH::DM], const SoftCall<SH::DM>& S, double& gt,
@@ -721,89 +749,66 @@ __device__ __forceinline__ void soft_channel(const Params& P, const SH& sh, cons
     const uint32_t mmask = h.mmask;
     const int n = sh.n();
     uint64_t acc = 1ull << 63;
-    int ae = 0, rows = 0;  // acc 2^(ae - 1022 rows - 63)
+    int ae = 0;  // acc 2^(ae - 1022 d - 63) once every row is in
     if (lookups) {
-        if (h.slow == 0u) {
+        const uint32_t slow = h.slow;
 #pragma unroll
-            for (int k = 0; k < SH::DM; ++k) {
-                if (sh.has(k) && !((mmask >> k) & 1u)) {
-                    const unsigned char* row = sh.row(blk, k);
-                    const double* e = reinterpret_cast<const double*>(row);
-                    int j = row[sh.tab_off() + S.q[k]];
-                    j += Prec<double>::le(e[j + 1], p[k]) ? 1 : 0;
-                    if (REC) bins[k] = min(j, n - 1);
-                    soft_factor(acc, ae, reinterpret_cast<const uint64_t*>(row + sh.dens_off())[j]);
-                }
-                if (k % 4 == 3) {  // four factors lose at most four leading bits
-                    const int z = sf_clz(acc);
-                    acc <<= z;
-                    ae -= z;
-                }
-            }
-            rows = sh.d() - __popc(mmask);
-        } else {
-            for (int k = 0; k < sh.d(); ++k) {
-                if ((mmask >> k) & 1u) continue;
+        for (int k = 0; k < SH::DM; ++k) {
+            if (sh.has(k) && !((mmask >> k) & 1u)) {
                 const unsigned char* row = sh.row(blk, k);
                 const double* e = reinterpret_cast<const double*>(row);
-                const double pk = S.p[k];
-                int j = row[sh.tab_off() + Prec<double>::cell(pk, sh.lshift())];
-                for (int s = 128; s > 0; s >>= 1)  // largest j with e[j] <= p
-                    if (j + s < n && Prec<double>::le(e[j + s], pk)) j += s;
-                if (REC) bins[k] = j;
+                int j = row[sh.tab_off() + S.q[k]];
+                j += Prec<double>::le(e[j + 1], p[k]) ? 1 : 0;
+                if ((slow >> k) & 1u) j = soft_search(e, j, n, p[k]);  // a cell of more than two bins
+                if (REC) bins[k] = min(j, n - 1);  // (entry n of the densities repeats the last)
                 soft_factor(acc, ae, reinterpret_cast<const uint64_t*>(row + sh.dens_off())[j]);
-                const int z = sf_clz(acc);
-                acc <<= z;
-                ae -= z;
-                ++rows;
             }
+            if (k % 8 == 7 || k == SH::DM - 1) sf_norm(acc, ae);
         }
     }
+    // den: Breit-Wigner denominators; G: p^(-4/5); F: the peak's factors
     const Sf one{1ull << 63, -63};
     Sf den = one, G = one, F = S.e0;
     double as = 0.0;
-    bool any_bw = false;
 #pragma unroll 1
     for (uint32_t s = 0; s < h.nslot; ++s) {
         const int k = h.sk[s] & 15;
         const double pk = S.p[k];
-        float xc;  // cell of the FP32 inverse map, a fraction of a cell low
+        float xc;  // cell of the FP32 inverse map
         if ((h.sk[s] >> 4) == MAP_BW) {
             const double dp = pk - h.c0[s];
-            den = sf_norm(sf_mul(den, sf_from_double(dp * dp + h.c1[s])));
-            any_bw = true;
-            xc = (atanf(sf_to_float(dp) * h.pinvG[s]) + h.pt0[s]) * h.pscale[s];
+            den = sf_mul(den, sf_from_double(dp * dp + h.c1[s]));
+            xc = (atan_start(sf_to_float(dp) * h.pinvG[s]) + h.pt0[s]) * h.pscale[s];
         } else {
-            if (with_f) F = sf_norm(sf_mul(F, sf_powm08(pk + h.c0[s])));
-            G = sf_norm(sf_mul(G, sf_unpack(S.W[k])));
+            if (with_f) F = sf_mul(F, sf_powm08(pk + h.c0[s]));
+            G = sf_mul(G, sf_unpack(S.W[k]));
             const uint64_t b = sf_bits(pk);
             const float lg = sf_lg2f((float)(((uint32_t)(b >> 29) & 0x7fffffu) | 0x800000u)) + (float)((int)((int64_t)b >> 52) - 1046);
-            // (p < 0, by rounding at a map's lower end, gives cell 0)
-            xc = sf_ex2f(0.2f * lg) * h.pscale[s];
+            xc = sf_ex2f(0.2f * lg) * h.pscale[s];  // (p < 0, by rounding at a map's lower end, gives cell 0)
         }
         if (with_f) {
             if (gauss_sum) as += sf_from_bits(S.E[k]);
-            else F = sf_norm(sf_mul(F, sf_unpack(S.E[k])));
+            else F = sf_mul(F, sf_unpack(S.E[k]));
         }
         if (lookups) {
             const unsigned char* row = sh.row(blk, k);
             const double* e = reinterpret_cast<const double*>(row);
             const int L = 1 << sh.lshift();
             int j = row[sh.tab_off() + min(max((int)(xc - 0.02f), 0), L)];
-            while (j < n - 1 && Prec<double>::le(e[j + 1], pk)) ++j;
-            if (REC) bins[k] = j;
+            j = soft_search(e, j, n, pk);
+            if (REC) bins[k] = min(j, n - 1);
             soft_factor(acc, ae, reinterpret_cast<const uint64_t*>(row + sh.dens_off())[j]);
-            const int z = sf_clz(acc);
-            acc <<= z;
-            ae -= z;
-            ++rows;
         }
     }
-    if (with_f && gauss_sum) F = sf_norm(sf_mul(F, sf_exp2(as - S.A)));
-    const Sf y = any_bw ? sf_rcp(den) : one;
-    const Sf a{acc, ae - 1022 * rows - 63};
-    gt = lookups ? sf_to_double(sf_norm(sf_mul(sf_mul(a, G), y))) : 0.0;
-    ft = with_f ? sf_to_double(sf_norm(sf_mul(F, y))) : 0.0;
+    Sf y = one;
+    if (h.bw) y = sf_rcp(sf_norm(den));
+    if (with_f && gauss_sum) F = sf_mul(sf_norm(F), sf_exp2(as - S.A));
+    gt = ft = 0.0;
+    if (lookups) {
+        sf_norm(acc, ae);
+        gt = sf_to_double(sf_norm(sf_mul(sf_mul(Sf{acc, ae - 1022 * sh.d() - 63}, G), y)));
+    }
+    if (with_f) ft = sf_to_double(sf_norm(sf_mul(sf_norm(F), y)));
 }
 
 // Integrand of a non-matching problem: loop over its own peaks.

@@ -52,9 +52,11 @@ struct EvalArgs {
 };
 
 // One compiled pass kernel pair (integration, generation): precision, calls
-// per thread, and the shape it is specialised for (D = NB = 0: any shape).
+// per thread, and the shape it is specialised for (D = NB = 0: any shape, or
+// any number of bins with d in dlo..dhi).
 struct PassVariant {
     int fp32, cpt, D, NB;
+    int dlo = 0, dhi = 0;
     int minb;  // CTAs per SM the kernel is compiled for (register cap), sizes its tile budget
     const char* family;  // kernel template name ("k_pass" or "k_union")
     int uni = 0;         // runs on the union interval tables (vamp_union.cu), not on staged tiles
@@ -64,7 +66,9 @@ struct PassVariant {
 
 void add_pass_variants_f32_generic(std::vector<PassVariant>& v);
 void add_pass_variants_f32_shapes(std::vector<PassVariant>& v);
+void add_pass_variants_f32_dims(std::vector<PassVariant>& v);
 void add_pass_variants_f64(std::vector<PassVariant>& v);
+void add_pass_variants_f64_dims(std::vector<PassVariant>& v);
 void add_pass_variants_union(std::vector<PassVariant>& v);
 
 // ---- interval tables of the union pass (vamp_union.cu) -----------------------
@@ -115,7 +119,9 @@ TilePlan plan_tiles(size_t S, int K, int dn, size_t fixed, size_t budget);
 // The pass kernel's, at two CTAs per SM (TILE_BUDGET) or `minb` CTAs per SM
 // of the current device.
 TilePlan pass_smem(const Params& P, int fp32, int minb = 2);
-// Candidate kernels for a shape: exact (D, NB) matches first, then generic;
+// Candidate kernels for a shape: exact (D, NB) matches first, then those of
+// its range of d (pseudo-stratified passes: the any-shape form, which alone
+// carries the cell code);
 // with the channel count K given (K > 0) and union_fits, the union kernels
 // after them (exact shape first).
 std::vector<const PassVariant*> pass_candidates(int fp32, int d, int n, int stratified = 0, int K = 0);

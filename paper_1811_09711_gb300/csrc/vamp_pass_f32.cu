@@ -1,4 +1,4 @@
-// FP32-eval pass kernels for any shape (d <= 16, n <= 256).
+// FP32-eval pass kernels for any shape (d <= 16, n <= 256): pseudo-stratified passes.
 #include "vamp_pass.cuh"
 
 namespace vamp {

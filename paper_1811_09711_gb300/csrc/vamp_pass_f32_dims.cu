@@ -1,0 +1,16 @@
+// FP32-eval pass kernels by range of d (any number of bins).
+#include "vamp_pass.cuh"
+
+namespace vamp {
+void add_pass_variants_f32_dims(std::vector<PassVariant>& v)
+{
+    v.push_back(make_variant_dims<float, 2, 1, 4>());
+    v.push_back(make_variant_dims<float, 2, 5, 8>());
+    v.push_back(make_variant_dims<float, 2, 9, 12>());
+    v.push_back(make_variant_dims<float, 2, 13, 16>());
+    v.push_back(make_variant_dims<float, 1, 1, 4>());
+    v.push_back(make_variant_dims<float, 1, 5, 8>());
+    v.push_back(make_variant_dims<float, 1, 9, 12>());
+    v.push_back(make_variant_dims<float, 1, 13, 16>());
+}
+}  // namespace vamp

@@ -123,11 +123,12 @@ void make_hdr(const vamp_map_desc& r, double weight, double zinv, int d, int lsh
             h.mmask |= 1u << r.coord[s];
             h.sk[q] = (uint8_t)(r.coord[s] | kind << 4);
             // cells of the row's table per unit of the FP32 inverse map, whose
-            // error (about 4e-7 / A) must stay below the 0.02 cells that the
+            // error (about 2e-6 / A) must stay below the 0.02 cells that the
             // lookup allows it; 0: the search starts at the first bin
             const double cells = (double)(1 << lshift);
             if (kind == MAP_BW) {
                 const double A = h.sp[s][SP_A];
+                h.bw = 1;
                 h.c0[q] = h.sp[s][SP_M];
                 h.c1[q] = h.sp[s][SP_G2];
                 h.gN *= h.sp[s][SP_GINVA];
@@ -389,7 +390,9 @@ std::vector<const PassVariant*> pass_candidates(int fp32, int d, int n, int stra
     std::call_once(once, [] {
         add_pass_variants_f32_generic(all);
         add_pass_variants_f32_shapes(all);
+        add_pass_variants_f32_dims(all);
         add_pass_variants_f64(all);
+        add_pass_variants_f64_dims(all);
         add_pass_variants_union(all);
     });
     const bool uni = K > 0 && union_fits(fp32, d, K, n, stratified);
@@ -403,7 +406,7 @@ std::vector<const PassVariant*> pass_candidates(int fp32, int d, int n, int stra
             continue;
         }
         if (v.D == d && v.NB == n && !stratified) exact.push_back(&v);
-        else if (v.D == 0 && v.NB == 0) generic.push_back(&v);
+        else if (v.D == 0 && v.NB == 0 && (stratified ? v.dhi == 0 : v.dlo <= d && d <= v.dhi)) generic.push_back(&v);
     }
     for (const PassVariant* v : generic) exact.push_back(v);
     for (const PassVariant* v : uexact) exact.push_back(v);

@@ -59,13 +59,19 @@ VAMP_HD double sf_from_bits(uint64_t b)
 #endif
 }
 
-VAMP_HD int sf_clz(uint64_t m)
+// Normalises m 2^e whose leading bit is among the upper 32.
+VAMP_HD void sf_norm(uint64_t& m, int& e)
 {
+    const uint32_t hi = (uint32_t)(m >> 32), lo = (uint32_t)m;
 #ifdef __CUDA_ARCH__
-    return __clzll((long long)m);
+    const int z = __clz((int)hi);
+    m = ((uint64_t)__funnelshift_l(lo, hi, z) << 32) | (lo << z);
 #else
-    return m ? __builtin_clzll(m) : 64;
+    const int z = __builtin_clz(hi);
+    m <<= z;
+    (void)lo;
 #endif
+    e -= z;
 }
 
 // High 64 bits of a b without the low halves' product: short of the true
@@ -78,8 +84,8 @@ VAMP_HD uint64_t sf_mulhi(uint64_t a, uint64_t b)
 
 VAMP_HD Sf sf_norm(Sf a)
 {
-    const int s = sf_clz(a.m);
-    return Sf{a.m << (s & 63), a.e - s};
+    sf_norm(a.m, a.e);
+    return a;
 }
 
 VAMP_HD Sf sf_mul(Sf a, Sf b) { return Sf{sf_mulhi(a.m, b.m), a.e + b.e + 64}; }
@@ -226,13 +232,16 @@ VAMP_HD Sf sf_powm08(double v)
     const uint64_t q = sf_mulhi(m, s5);                       // X s^5 2^-h, Q5.59
     const int64_t d = (int64_t)((1ull << (59 - h)) - q);
     const int64_t r = (int64_t)((uint64_t)d << (3 + h));      // Q0.62, |r| < 2^43
-    // 0.8 r = r - r / 5 (the constant is 2^34 / 5), 0.72 r^2
-    const int64_t r5 = (int64_t)((uint64_t)sf_scale(3435973837u, r, 32)) >> 2;
-    const int32_t rh = (int32_t)(r >> 20);
-    const uint32_t r2 = (uint32_t)(((int64_t)rh * rh) >> 22);
-    const int64_t c = r - r5 + (int64_t)(((uint64_t)r2 * 3092376453u) >> 32);
-    const uint64_t z = s4 + (uint64_t)sf_scale((uint32_t)(s4 >> 32), c, 30) +
-                       (uint64_t)((int64_t)((int64_t)(uint32_t)s4 * (int64_t)(int32_t)(c >> 30)) >> 32);
+    // c = 0.8 r + 0.72 r^2 in Q0.64 (|c| < 2^45): 0.8 r = r - r / 5 with 2^34 / 5, r^2 from the upper bits
+    const uint32_t rl = (uint32_t)r;
+    const int32_t rh = (int32_t)(r >> 32), rm = (int32_t)(r >> 20);
+    const int64_t r5 = (int64_t)(((uint64_t)rl * 3435973837u >> 32) + (uint64_t)((int64_t)rh * 3435973837ll));  // 4 r / 5
+    const uint32_t r2 = (uint32_t)(((int64_t)rm * rm) >> 20);
+    const int64_t c = 4 * r - r5 + (int64_t)(((uint64_t)r2 * 3092376453u) >> 32);
+    const int32_t ch = (int32_t)(c >> 32);
+    const uint32_t zh = (uint32_t)(s4 >> 32), zl = (uint32_t)s4;
+    const uint64_t z = s4 + (uint64_t)((int64_t)ch * (int64_t)(uint64_t)zh) + (((uint64_t)zh * (uint32_t)c) >> 32) +
+                       (uint64_t)((int64_t)((int64_t)ch * (int64_t)(uint64_t)zl) >> 32);
     return sf_norm(Sf{z, -60 - 4 * a});
 }
 
