@@ -451,10 +451,7 @@ vamp_status enqueue_pass(vamp_ctx* c, int64_t n_calls, uint32_t iteration, cudaE
         c->tuned = 1;
     }
     const Params& P = c->prm;
-    VAMP_CK(c, cudaMemsetAsync(P.D, 0, (size_t)c->K * c->d * c->n * 8, c->stream));
-    VAMP_CK(c, cudaMemsetAsync(P.csum, 0, (size_t)2 * c->K * 8, c->stream));
-    if (P.stratified) VAMP_CK(c, cudaMemsetAsync(P.cellsum, 0, (size_t)max_cells * 8, c->stream));
-    VAMP_CK(c, vamp::launch_begin_pass(P, n_calls, c->stream));
+    VAMP_CK(c, vamp::launch_begin_pass(P, n_calls, c->stream, 1, max_cells));
     if (e0) VAMP_CK(c, cudaEventRecord(e0, c->stream));
     VAMP_CK(c, c->var->launch(P, 0, pass_args(c, iteration), c->grid_pass, c->smem_pass, c->stream));
     if (e1) VAMP_CK(c, cudaEventRecord(e1, c->stream));

@@ -120,6 +120,7 @@ struct Scalars {
     long long gen_take;              // taken from this batch
     long long gen_used;              // calls consumed in this batch
     long long gen_over;              // overweights among taken
+    double wmax_cut;                 // w_max that this batch was accepted against
     // history of passes for the combination of iterations
     int32_t n_hist;
     int32_t pad1;
@@ -131,6 +132,7 @@ struct Scalars {
 // All pointers and sizes a kernel needs (passed by value).
 struct Params {
     int d, K, n, P;
+    int fp32;              // evaluation precision of the passes
     uint32_t map_any, pow_any;  // bit k: some channel has a Breit-Wigner or power-law map (a power-law map) on k
     int gauss_sum;         // the Gaussian factor of one coordinate can leave the packed range: exponents are summed
     int matching;          // peaks are the channels' maps (integrand fused into the channel loop)

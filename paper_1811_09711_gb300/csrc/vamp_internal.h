@@ -168,7 +168,8 @@ cudaError_t launch_pass_multi(int fp32, int minb, const MultiArgs& M, int grid, 
 // strat: the form that also runs pseudo-stratified instances
 const void* pass_multi_kernel(int fp32, int minb, int strat = 0);
 
-cudaError_t launch_begin_pass(const Params& P, int64_t N, cudaStream_t s);
+// clear: also zero the pass accumulators, with `cells` cell sums
+cudaError_t launch_begin_pass(const Params& P, int64_t N, cudaStream_t s, int clear = 0, int64_t cells = 0);
 cudaError_t launch_finish_pass(const Params& P, int combine, cudaStream_t s);
 cudaError_t launch_strat_q(const Params& P, cudaStream_t s);  // stratified passes, before finish
 cudaError_t launch_derive(const Params& P, cudaStream_t s);

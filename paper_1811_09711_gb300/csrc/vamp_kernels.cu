@@ -1,7 +1,7 @@
 // vamp_kernels.cu -- the small kernels around the pass kernel (vamp_pass.cuh):
 //
 //   k_begin_pass      integer call allocation N_c, prefix P_c (§3.4); cells of a
-//                     pseudo-stratified pass (§3.3)
+//                     pseudo-stratified pass (§3.3); clears the accumulators
 //   k_strat_q         Σ over a channel's cells of the squared cell sums (§3.3)
 //   k_finish_pass     per-channel means/variances, pass result, combination
 //   k_pass_result     pass result into a caller's device array (asynchronous pass)
@@ -9,11 +9,13 @@
 //                     with the channel equivalences pooled in (§3.5)
 //   k_update_alpha    channel-weight update (Eq. 25)
 //   k_derive          lookup-block rows: densities 1/(n Δx), cell tables, FP32 copies
-//   k_gen_prepare / k_gen_scan / k_gen_copy / k_gen_end   generation bookkeeping
+//   k_gen_prepare / k_gen_scan / k_gen_copy   generation bookkeeping
 //   k_eval<T>         per-call diagnostics for parity tests
 //   k_batch_*         the same steps for every instance of a batch or server tick
 #include "vamp_device.cuh"
 #include "vamp_internal.h"
+
+#include <algorithm>
 
 namespace vamp {
 
@@ -37,21 +39,74 @@ __device__ int64_t strat_cells_per_axis(int64_t N, int d)
     return lo;
 }
 
+// Inclusive scan of v over the block (all threads; at most 1024), and the sum
+// over the block through `total`.  tmp: 33 words of shared memory.
+template <typename V>
+__device__ __forceinline__ V block_scan(V v, V* tmp, V* total)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const V y = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += y;
+    }
+    __syncthreads();  // tmp is free again
+    if (lane == 31) tmp[wid] = v;
+    __syncthreads();
+    if (wid == 0) {
+        V w = lane < nw ? tmp[lane] : V(0);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const V y = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += y;
+        }
+        if (lane < nw) tmp[lane] = w;
+        if (lane == nw - 1) tmp[32] = w;
+    }
+    __syncthreads();
+    *total = tmp[32];
+    return v + (wid > 0 ? tmp[wid - 1] : V(0));
+}
+
+// Sum over the block in a fixed order, to every thread.
+__device__ __forceinline__ double block_sum(double v, double* tmp)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();
+    if (lane == 0) tmp[wid] = v;
+    __syncthreads();
+    double s = 0.0;
+    for (int q = 0; q < nw; ++q) s += tmp[q];
+    return s;
+}
+
+__device__ __forceinline__ double lanes_sum(double v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Called by every thread of one block (a multiple of 32 threads), a channel a
+// thread: with one thread walking the channels the allocation of K = 64 took
+// 12 us, the pass results 35 and the weights 19.
 __device__ void begin_pass_dev(const Params& P, int64_t N)
 {
-    {
-        int64_t acc = 0, cells = 0;
-        P.Pc[0] = 0;
-        if (P.stratified) P.coff[0] = 0;
-        for (int c = 0; c < P.K; ++c) {
-            int64_t nc = 0;
+    __shared__ long long tmp[33];
+    long long acc = 0, cells = 0;
+    for (int c0 = 0; c0 < P.K; c0 += blockDim.x) {
+        const int c = c0 + (int)threadIdx.x;
+        long long nc = 0, m = 1, s = 0, C = 1;
+        if (c < P.K) {
             if (P.alpha[c] > 0.0) {
-                nc = (int64_t)floor(P.alpha[c] * (double)N);
+                nc = (long long)floor(P.alpha[c] * (double)N);
                 if (nc < P.n_min) nc = P.n_min;
             }
             if (P.stratified) {
                 // whole cells: n_r per axis, C = n_r^d cells, s = floor(N_c / C)
-                int64_t m = 1, C = 1, s = nc;
+                s = nc;
                 if (nc >= 2) {
                     m = strat_cells_per_axis(nc, P.d);
                     for (int k = 0; k < P.d; ++k) C *= m;
@@ -60,61 +115,82 @@ __device__ void begin_pass_dev(const Params& P, int64_t N)
                 nc = s * C;
                 P.nr[c] = m;
                 P.spc[c] = s;
-                cells += C;
-                P.coff[c + 1] = cells;
             }
             P.Nc[c] = nc;
-            acc += nc;
-            P.Pc[c + 1] = acc;
         }
+        long long tot;
+        const long long incl = block_scan(c < P.K ? nc : 0ll, tmp, &tot);
+        if (c < P.K) P.Pc[c + 1] = acc + incl;
+        acc += tot;
+        if (P.stratified) {
+            const long long ci = block_scan(c < P.K ? C : 0ll, tmp, &tot);
+            if (c < P.K) P.coff[c + 1] = cells + ci;
+            cells += tot;
+        }
+    }
+    if (threadIdx.x == 0) {
+        P.Pc[0] = 0;
+        if (P.stratified) P.coff[0] = 0;
         P.sc->n_total = acc;
         P.sc->wmax_bits = 0ull;
     }
 }
 
 // Stratified passes: Q_c = Σ over the channel's cells of the squared cell
-// sums, one 256-thread block per channel, fixed-order reduction (the same
-// for a context and for an instance of a batch).
-__device__ void strat_q_channel(const Params& P, int c)
+// sums (Qc is zero before), `parts` blocks of 256 threads per channel: one
+// block alone took 211 us for the 5e5 cells of a 1e6-call channel.
+constexpr int STRAT_PARTS = 32;
+
+__device__ void strat_q_channel(const Params& P, int c, int part, int parts)
 {
-    __shared__ double part[256];
-    const int64_t a = P.coff[c], b = P.coff[c + 1];
+    __shared__ double tmp[33];
+    const int64_t a = P.coff[c], len = P.coff[c + 1] - a;
+    const int64_t lo = a + len * part / parts, hi = a + len * (part + 1) / parts;
     double s = 0.0;
-    for (int64_t q = a + threadIdx.x; q < b; q += blockDim.x) {
+    for (int64_t q = lo + threadIdx.x; q < hi; q += blockDim.x) {
         const double v = P.cellsum[q];
         s += v * v;
     }
-    part[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) part[threadIdx.x] += part[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) P.Qc[c] = part[0];
+    s = block_sum(s, tmp);
+    if (threadIdx.x == 0 && hi > lo) atomicAdd(&P.Qc[c], s);
 }
 
 __global__ void k_strat_q(Params P)
 {
-    strat_q_channel(P, blockIdx.x);
+    strat_q_channel(P, blockIdx.x, blockIdx.y, gridDim.y);
 }
 
-__global__ void k_begin_pass(Params P, int64_t N)
+// Block 0 allocates; with clear != 0 all blocks clear the pass accumulators
+// (and `cells` cell sums).
+__global__ void k_begin_pass(Params P, int64_t N, int clear, int64_t cells)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) begin_pass_dev(P, N);
+    if (clear) {
+        const int64_t nd = (int64_t)P.K * P.d * P.n, t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x,
+                      nt = (int64_t)gridDim.x * blockDim.x;
+        for (int64_t q = t0; q < nd; q += nt) P.D[q] = 0.0;
+        for (int64_t q = t0; q < 2 * P.K; q += nt) P.csum[q] = 0.0;
+        if (P.stratified) {
+            for (int64_t q = t0; q < cells; q += nt) P.cellsum[q] = 0.0;
+            for (int64_t q = t0; q < P.K; q += nt) P.Qc[q] = 0.0;
+        }
+    }
+    if (blockIdx.x == 0) begin_pass_dev(P, N);
 }
 
 // ---------------------------------------------------------------------------
 // pass result (Eqs. 10, 11 per channel on shifted sums; Eq. 23; R8, R9)
 // ---------------------------------------------------------------------------
-// Called by every thread of one block: per-channel values in parallel, then
-// thread 0 sums them in channel order (the order of the scalar form).
+// Called by every thread of one block: per-channel values and their sums by
+// all, the combination of the passes by the first warp.
 __device__ void finish_pass_dev(const Params& P, int combine)
 {
+    __shared__ double tmp[33];
     Scalars* sc = P.sc;
+    double I = 0.0, V = 0.0;
     for (int c = threadIdx.x; c < P.K; c += blockDim.x) {
         const int64_t nci = P.Nc[c];
         if (nci == 0) { P.Ic[c] = P.Vc[c] = P.Wc[c] = 0.0; P.shift[c] = 0.0; continue; }
-        const double Nc = (double)nci;
+        const double Nc = (double)nci, al = P.alpha[c];
         const double m1 = P.csum[2 * c] / Nc, m2 = P.csum[2 * c + 1] / Nc;
         const double Ic = P.shift[c] + m1;
         double Vv = 0.0;
@@ -130,54 +206,55 @@ __device__ void finish_pass_dev(const Params& P, int combine)
         P.Vc[c] = Vv;
         P.Wc[c] = (m2 - m1 * m1) + Ic * Ic;
         P.shift[c] = Ic;  // R13: the next pass's sums are taken about this mean
+        I += al * Ic;
+        V += al * al * Vv / Nc;
     }
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    double I = 0.0, V = 0.0;
-    for (int c = 0; c < P.K; ++c) {
-        if (P.Nc[c] == 0) continue;
-        I += P.alpha[c] * P.Ic[c];
-        V += P.alpha[c] * P.alpha[c] * P.Vc[c] / (double)P.Nc[c];
-    }
-    const double wmax = __longlong_as_double((long long)sc->wmax_bits);
-    sc->wmax_gen = wmax;
-    const int h = sc->n_hist;
-    if (h < 1024) {
+    I = block_sum(I, tmp);
+    V = block_sum(V, tmp);
+    if (threadIdx.x >= 32) return;
+    const int lane = threadIdx.x;
+    // the passes so far and this one
+    const int h = sc->n_hist, nh = h < 1024 ? h + 1 : h;
+    if (lane == 0 && h < 1024) {
         sc->hist_I[h] = I;
         sc->hist_V[h] = V;
         sc->hist_comb[h] = combine;
         sc->n_hist = h + 1;
     }
+    __syncwarp();
     // inverse-variance combination of the flagged passes
-    int cnt = 0, nzero = 0;
-    double zI = 0.0;
-    for (int q = 0; q < sc->n_hist; ++q) {
+    double cnt = 0.0, nzero = 0.0, zI = 0.0, sw = 0.0, swi = 0.0;
+    for (int q = lane; q < nh; q += 32) {
         if (!sc->hist_comb[q]) continue;
-        ++cnt;
-        if (sc->hist_V[q] <= 0.0) { ++nzero; zI += sc->hist_I[q]; }
+        const double hI = sc->hist_I[q], hV = sc->hist_V[q];
+        cnt += 1.0;
+        if (hV <= 0.0) { nzero += 1.0; zI += hI; }
+        else { const double iv = 1.0 / hV; sw += iv; swi += hI / hV; }
     }
+    cnt = lanes_sum(cnt);
     double cI = 0.0, cS = 0.0, chi = 0.0;
-    if (cnt > 0 && nzero > 0) {
-        cI = zI / nzero;
-    } else if (cnt > 0) {
-        double sw = 0.0, swi = 0.0;
-        for (int q = 0; q < sc->n_hist; ++q) {
-            if (!sc->hist_comb[q]) continue;
-            sw += 1.0 / sc->hist_V[q];
-            swi += sc->hist_I[q] / sc->hist_V[q];
-        }
-        cI = swi / sw;
-        cS = sqrt(1.0 / sw);
-        if (cnt > 1) {
-            double ch = 0.0;
-            for (int q = 0; q < sc->n_hist; ++q) {
-                if (!sc->hist_comb[q]) continue;
-                const double dI = sc->hist_I[q] - cI;
-                ch += dI * dI / sc->hist_V[q];
+    if (cnt > 0.0) {
+        nzero = lanes_sum(nzero);
+        if (nzero > 0.0) {
+            cI = lanes_sum(zI) / nzero;
+        } else {
+            sw = lanes_sum(sw);
+            cI = lanes_sum(swi) / sw;
+            cS = sqrt(1.0 / sw);
+            if (cnt > 1.0) {
+                double ch = 0.0;
+                for (int q = lane; q < nh; q += 32) {
+                    if (!sc->hist_comb[q]) continue;
+                    const double dI = sc->hist_I[q] - cI;
+                    ch += dI * dI / sc->hist_V[q];
+                }
+                chi = lanes_sum(ch) / (cnt - 1.0);
             }
-            chi = ch / (double)(cnt - 1);
         }
     }
+    if (lane != 0) return;
+    const double wmax = __longlong_as_double((long long)sc->wmax_bits);
+    sc->wmax_gen = wmax;
     sc->res[0] = I;
     sc->res[1] = V;
     sc->res[2] = wmax;
@@ -207,13 +284,14 @@ __global__ void k_pass_result(Params P, double* out)
 // ---------------------------------------------------------------------------
 // lookup blocks of one grid row (Eq. 12 densities, FP32 copies, cell tables)
 // ---------------------------------------------------------------------------
+// One warp derives grid row `row` from its edges e64 (global or shared memory).
+// q0: n+1 ints of warp scratch.
 template <typename T>
 __device__ __forceinline__ void derive_row_t(const Params& P, const BlkLayout& L, unsigned char* lk, int row,
-                                             int lane, int nl)
+                                             int lane, const double* e64, int* q0)
 {
     const int n = P.n, d = P.d;
     const int c = row / d, k = row % d;
-    const double* e64 = P.edges64 + (size_t)row * (n + 1);
     unsigned char* r = lk + (size_t)c * L.bytes + L.H + (size_t)k * L.R;
     T* e = reinterpret_cast<T*>(r);
     T* dnr = reinterpret_cast<T*>(r + L.Es * sizeof(T));
@@ -232,8 +310,11 @@ __device__ __forceinline__ void derive_row_t(const Params& P, const BlkLayout& L
             sp = h->sp[s];
         }
     }
-    for (int j = lane; j <= n; j += nl) {
-        double v = e64[j];
+    const bool over_x = sizeof(T) == 8 && kind != MAP_ID;
+    const int Lc = 1 << L.lshift;
+    for (int j = lane; j <= n; j += 32) {
+        const double x = e64[j];
+        double v = x;
         if (kind == MAP_BW) {
             v = sp[SP_M] + sp[SP_G] * Prec<double>::tan_(sp[SP_A] * v - sp[SP_T0]);
         } else if (kind == MAP_POW) {
@@ -241,29 +322,36 @@ __device__ __forceinline__ void derive_row_t(const Params& P, const BlkLayout& L
             v = v4 * v;
             if (v < Prec<double>::tiny()) v = Prec<double>::tiny();
         }
-        e[j] = (T)(v > 0.0 ? v : 0.0);
+        const T ev = (T)(v > 0.0 ? v : 0.0);
+        e[j] = ev;
+        // first cell boundary q/L at or above the edge (over x in the FP64 rows
+        // of mapped coordinates; scaling by L is exact)
+        const double tq = ceil((over_x ? x : (double)ev) * (double)Lc);
+        q0[j] = tq > (double)(Lc + 1) ? Lc + 1 : (int)tq;
         const int jb = j < n ? j : n - 1;  // entry n repeats bin n-1
-        const double dens = 1.0 / ((double)n * (e64[jb + 1] - e64[jb]));
-        if constexpr (sizeof(T) == 8) reinterpret_cast<uint64_t*>(dnr)[j] = sf_pack_double(dens);
-        else dnr[j] = (T)dens;
-    }
-    __syncwarp();
-    // tb[q] = largest j in [0, n-1] with e[j] <= q/L, for q = 0..L (over x
-    // in the FP64 rows of mapped coordinates)
-    const int Lc = 1 << L.lshift;
-    const bool over_x = sizeof(T) == 8 && kind != MAP_ID;
-    for (int q = lane; q <= Lc; q += nl) {
-        const T xq = (T)q / (T)Lc;
-        int lo = 0, hi = n - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if ((over_x ? (T)e64[mid] : e[mid]) <= xq) lo = mid; else hi = mid - 1;
+        const double dx = (double)n * (e64[jb + 1] - e64[jb]);
+        if constexpr (sizeof(T) == 8) {
+            // 1 / (n Δx), rounded to 53 bits (a subnormal Δx as the division has it)
+            reinterpret_cast<uint64_t*>(dnr)[j] =
+                dx >= 2.3e-308 ? sf_pack(sf_norm(sf_rcp(sf_from_double(dx)))) : sf_pack_double(1.0 / dx);
+        } else {
+            dnr[j] = (T)(1.0 / dx);
         }
-        tb[q] = (unsigned char)lo;
     }
     __syncwarp();
+    // tb[q] = largest j in [0, n-1] with edge j <= q/L, for q = 0..L: bin j
+    // takes the boundaries from its own edge's up to the next edge's; span =
+    // the most edges (of 1..n-1) inside one cell
     int span = 0;
-    for (int q = lane; q < Lc; q += nl) span = max(span, (int)tb[q + 1] - (int)tb[q]);
+    for (int j = lane; j < n; j += 32) {
+        const int a = j == 0 ? 0 : q0[j], b = j == n - 1 ? Lc + 1 : min(q0[j + 1], Lc + 1);
+        for (int q = a; q < b; ++q) tb[q] = (unsigned char)j;
+        if (j > 0 && a >= 1 && a <= Lc) {
+            int run = 1;
+            while (j + run <= n - 1 && q0[j + run] == a) ++run;
+            span = max(span, run);
+        }
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) span = max(span, __shfl_xor_sync(0xffffffffu, span, o));
     if (lane == 0) {
@@ -273,6 +361,14 @@ __device__ __forceinline__ void derive_row_t(const Params& P, const BlkLayout& L
         if (span > 1 && !over_x) atomicOr(slow, 1u << k);
         else atomicAnd(slow, ~(1u << k));
     }
+    __syncwarp();
+}
+
+// A context's passes read the blocks of its own precision only.
+__device__ __forceinline__ void derive_row(const Params& P, int row, int lane, const double* e64, int* q0)
+{
+    if (P.fp32) derive_row_t<float>(P, P.lay32, P.lk32, row, lane, e64, q0);
+    else derive_row_t<double>(P, P.lay64, P.lk64, row, lane, e64, q0);
 }
 
 // The forms of α_c that the pass kernels read beside alpha[c].
@@ -282,19 +378,15 @@ __device__ __forceinline__ void store_alpha(const Params& P, int c, double a)
     P.alphaN[c] = a * reinterpret_cast<const ChanHdr<double>*>(P.lk64 + (size_t)c * P.lay64.bytes)->gN;
 }
 
-__device__ __forceinline__ void derive_row(const Params& P, int row, int lane)
-{
-    derive_row_t<double>(P, P.lay64, P.lk64, row, lane, 32);
-    derive_row_t<float>(P, P.lay32, P.lk32, row, lane, 32);
-}
-
 __global__ void k_derive(Params P)
 {
+    extern __shared__ int dq0[];
     const int rows = P.K * P.d;
     const int lane = threadIdx.x & 31;
+    int* q0 = dq0 + (threadIdx.x >> 5) * (P.n + 1);
     const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int nw = gridDim.x * (blockDim.x >> 5);
-    for (int row = w; row < rows; row += nw) derive_row(P, row, lane);
+    for (int row = w; row < rows; row += nw) derive_row(P, row, lane, P.edges64 + (size_t)row * (P.n + 1), q0);
     if (blockIdx.x == 0)
         for (int c = threadIdx.x; c < P.K; c += blockDim.x) store_alpha(P, c, P.alpha[c]);
 }
@@ -302,7 +394,21 @@ __global__ void k_derive(Params P)
 // ---------------------------------------------------------------------------
 // rebinning, one warp per (channel, axis) row (Eqs. 14, 15; R2-R4)
 // ---------------------------------------------------------------------------
-// One warp rebins grid row `row` of P; ws = 4n+2 doubles of warp scratch.
+// ((r - 1) / ln r)^a for r in (0, 1): logarithms and powers on 64-bit mantissas
+// (an FP64 log and pow are some 150 operations of the FP64 pipe a bin, half of
+// the rebinning of the collider's 896 rows).  Near 1, where log r is small
+// against its error there, the FP64 log.
+__device__ __forceinline__ double rebin_measure(double r, double a)
+{
+    const double lr = r > 0.999 ? log(r) : sf_log2(r) * 0.6931471805599453;
+    const double v = (r - 1.0) / lr;
+    return sf_to_double(sf_norm(sf_exp2(a * sf_log2(v))));
+}
+
+// Doubles of warp scratch of refine_row_dev.
+__host__ __device__ constexpr int refine_scratch(int n) { return 5 * n + 4; }
+
+// One warp rebins grid row `row` of P; ws = refine_scratch(n) doubles.
 __device__ void refine_row_dev(const Params& P, int row, int lane, double* ws)
 {
     const int n = P.n;
@@ -310,6 +416,7 @@ __device__ void refine_row_dev(const Params& P, int row, int lane, double* ws)
     double* m = Dj + n;
     double* C = m + n;          // n+1
     double* eo = C + n + 1;     // n+1
+    double* en = eo + n + 1;    // n+1
     const double* Din = P.D + (size_t)row * n;
     double* e = P.edges64 + (size_t)row * (n + 1);
     for (int j = lane; j < n; j += 32) Dj[j] = Din[j];
@@ -348,30 +455,38 @@ __device__ void refine_row_dev(const Params& P, int row, int lane, double* ws)
         for (int j = lane; j < n; j += 32) Dj[j] = m[j];
         __syncwarp();
     }
-    for (int j = lane; j < n; j += 32) Dj[j] = sqrt(Dj[j]); // ω_j
-    __syncwarp();
     double S = 0.0;
-    if (lane == 0)
-        for (int j = 0; j < n; ++j) S += Dj[j];
-    S = __shfl_sync(0xffffffffu, S, 0);
-    if (!(S > 0.0)) return;  // axis kept (R2); lookup blocks unchanged
     for (int j = lane; j < n; j += 32) {
-        const double r = Dj[j] / S;
-        double mj;
-        if (r == 0.0) mj = 0.0;
-        else if (fabs(r - 1.0) < 1e-12) mj = 1.0;
-        else mj = pow((r - 1.0) / log(r), P.grid_alpha);
-        m[j] = mj;
+        const double w = sqrt(Dj[j]);  // ω_j
+        Dj[j] = w;
+        S += w;
     }
-    __syncwarp();
+    S = lanes_sum(S);
+    if (!(S > 0.0)) return;  // axis kept (R2); lookup blocks unchanged
+    // m_j and its cumulative, 32 bins at a time
     double M = 0.0;
-    if (lane == 0) {
-        C[0] = 0.0;
-        for (int j = 0; j < n; ++j) C[j + 1] = C[j] + m[j];
-        M = C[n];
+    if (lane == 0) C[0] = 0.0;
+    for (int j0 = 0; j0 < n; j0 += 32) {
+        const int j = j0 + lane;
+        double mj = 0.0;
+        if (j < n) {
+            const double r = Dj[j] / S;
+            if (r == 0.0) mj = 0.0;
+            else if (fabs(r - 1.0) < 1e-12) mj = 1.0;
+            else mj = rebin_measure(r, P.grid_alpha);
+            m[j] = mj;
+        }
+        double v = mj;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double y = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += y;
+        }
+        v += M;
+        if (j < n) C[j + 1] = v;
+        M = __shfl_sync(0xffffffffu, v, 31);
     }
     __syncwarp();
-    M = __shfl_sync(0xffffffffu, M, 0);
     if (!(M > 0.0)) return;
     for (int i = lane; i <= n; i += 32) {
         double ne;
@@ -389,9 +504,10 @@ __device__ void refine_row_dev(const Params& P, int row, int lane, double* ws)
             ne = __dadd_rn(eo[j - 1], __dmul_rn(fr, __dsub_rn(eo[j], eo[j - 1])));
         }
         e[i] = ne;
+        en[i] = ne;
     }
     __syncwarp();
-    derive_row(P, row, lane);
+    derive_row(P, row, lane, en, reinterpret_cast<int*>(Dj));  // n + 1 ints over Dj and m
 }
 
 __global__ void __launch_bounds__(REFINE_WARPS * 32) k_refine(Params P)
@@ -400,37 +516,34 @@ __global__ void __launch_bounds__(REFINE_WARPS * 32) k_refine(Params P)
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int row = blockIdx.x * REFINE_WARPS + wid;
     if (row >= P.K * P.d) return;
-    refine_row_dev(P, row, lane, rs + (size_t)wid * (4 * P.n + 2));
+    refine_row_dev(P, row, lane, rs + (size_t)wid * refine_scratch(P.n));
 }
 
 // ---------------------------------------------------------------------------
 // channel weights (Eq. 25 with R5)
 // ---------------------------------------------------------------------------
-// Called by every thread of one block: the channel terms α_c ω_c^β in
-// parallel (kept in Acum), the sums SU, MU and the normalisation by thread 0
-// in channel order (the order of the scalar form).
+// Called by every thread of one block, a channel a thread (Acum holds the
+// terms α_c ω_c^β and then the new weights between the sums).
 __device__ void update_alpha_dev(const Params& P)
 {
-    __shared__ double red[2];
+    __shared__ double tmp[33];
     const int K = P.K;
     auto omega = [&](int c) { return P.omega_mode ? P.Wc[c] : P.Vc[c]; };
-    auto live = [&](int c) { return P.alpha[c] > 0.0 && P.Nc[c] > 0 && omega(c) > 0.0; };
-    for (int c = threadIdx.x; c < K; c += blockDim.x)
-        P.Acum[c] = live(c) ? P.alpha[c] * pow(omega(c), P.beta) : 0.0;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double SU = 0.0, MU = 0.0;
-        for (int c = 0; c < K; ++c) {
-            if (live(c)) {
-                SU += P.Acum[c];
-                MU += P.alpha[c];
-            }
+    double SU = 0.0, MU = 0.0;
+    for (int c = threadIdx.x; c < K; c += blockDim.x) {
+        const double a = P.alpha[c], w = omega(c);
+        double u = 0.0;
+        if (a > 0.0 && P.Nc[c] > 0 && w > 0.0) {
+            // ω^β (pow where ω is beyond a normal number)
+            u = a * (w >= 2.3e-308 && w < INFINITY ? sf_to_double(sf_norm(sf_exp2(P.beta * sf_log2(w)))) : pow(w, P.beta));
+            SU += u;
+            MU += a;
         }
-        red[0] = SU;
-        red[1] = MU;
+        P.Acum[c] = u;
     }
-    __syncthreads();
-    const double SU = red[0], MU = red[1];
+    SU = block_sum(SU, tmp);
+    MU = block_sum(MU, tmp);
+    double tot = 0.0;
     for (int c = threadIdx.x; c < K; c += blockDim.x) {
         double a = P.alpha[c];
         if (a > 0.0 && P.Nc[c] > 0) {
@@ -438,15 +551,9 @@ __device__ void update_alpha_dev(const Params& P)
             else if (P.Ic[c] == 0.0) a = 0.0;  // every call of the channel gave w = 0
         }
         P.Acum[c] = a;  // new weights, normalised below
+        tot += a;
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double tot = 0.0;
-        for (int c = 0; c < K; ++c) tot += P.Acum[c];
-        red[0] = tot;
-    }
-    __syncthreads();
-    const double tot = red[0];
+    tot = block_sum(tot, tmp);
     for (int c = threadIdx.x; c < K; c += blockDim.x) {
         if (tot > 0.0) P.alpha[c] = P.Acum[c] / tot;
         store_alpha(P, c, P.alpha[c]);
@@ -463,36 +570,44 @@ __global__ void k_update_alpha(Params P)
 // ---------------------------------------------------------------------------
 __global__ void k_gen_prepare(Params P)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    __shared__ double tmp[33];
     double acc = 0.0;
-    for (int c = 0; c < P.K; ++c) { acc += P.alpha[c]; P.Acum[c] = acc; }
-    P.sc->gen_bmax_bits = 0ull;
+    for (int c0 = 0; c0 < P.K; c0 += blockDim.x) {
+        const int c = c0 + (int)threadIdx.x;
+        double tot;
+        const double v = block_scan(c < P.K ? P.alpha[c] : 0.0, tmp, &tot);
+        if (c < P.K) P.Acum[c] = acc + v;
+        acc += tot;
+    }
+    if (threadIdx.x == 0) P.sc->gen_bmax_bits = 0ull;
 }
 
-// Exclusive prefix of the per-chunk counts, how many to take, calls used.
+// Exclusive prefix of the per-chunk counts, how many to take, calls used; the
+// batch's maximum weight into w_max for the next batch (wmax_cut keeps the
+// bound that this batch was accepted against).
 __global__ void k_gen_scan(Params P, PassArgs G, int64_t remaining)
 {
-    __shared__ long long part[1024];
+    __shared__ long long tmp[33];
     const int tid = threadIdx.x, nt = blockDim.x;
     const int nb = (int)G.nchunks;
     const int per = (nb + nt - 1) / nt;
-    const int b0 = tid * per, b1 = min(nb, b0 + per);
+    const int b0 = min(nb, tid * per), b1 = min(nb, b0 + per);
     long long s = 0;
     for (int b = b0; b < b1; ++b) s += G.counts[b];
-    part[tid] = s;
-    __syncthreads();
+    long long total;
+    long long off = block_scan(s, tmp, &total) - s;
+    const long long take = total < remaining ? total : remaining;
     if (tid == 0) {
-        long long a = 0;
-        for (int q = 0; q < nt; ++q) { const long long v = part[q]; part[q] = a; a += v; }
-        P.sc->gen_total = a;
-        const long long take = a < remaining ? a : remaining;
-        P.sc->gen_take = take;
-        P.sc->gen_over = 0;
-        P.sc->gen_used = G.batch;
+        Scalars* sc = P.sc;
+        sc->gen_total = total;
+        sc->gen_take = take;
+        sc->gen_over = 0;
+        if (!(take == remaining && take > 0)) sc->gen_used = G.batch;
+        const double bm = __longlong_as_double((long long)sc->gen_bmax_bits), cut = sc->wmax_gen;
+        sc->wmax_cut = cut;
+        if (bm > cut) sc->wmax_gen = bm;
+        sc->gen_bmax_bits = 0ull;
     }
-    __syncthreads();
-    long long off = part[tid];
-    const long long take = P.sc->gen_take;
     for (int b = b0; b < b1; ++b) {
         const long long cnt = G.counts[b];
         G.offsets[b] = off;
@@ -515,7 +630,7 @@ __global__ void k_gen_copy(Params P, PassArgs G, unsigned char* out)
     const unsigned long long* src =
         reinterpret_cast<const unsigned long long*>(G.staging + (int64_t)b * G.chunk * G.rec_bytes);
     unsigned long long* dst = reinterpret_cast<unsigned long long*>(out + off * G.rec_bytes);
-    const double wmax = P.sc->wmax_gen;
+    const double wmax = P.sc->wmax_cut;
     int over = 0;
     for (long long q = threadIdx.x; q < ncopy * words; q += blockDim.x) dst[q] = src[q];
     for (long long r = threadIdx.x; r < ncopy; r += blockDim.x) {
@@ -524,15 +639,6 @@ __global__ void k_gen_copy(Params P, PassArgs G, unsigned char* out)
         over += (fabs(w) > wmax);
     }
     if (over) atomicAdd(reinterpret_cast<unsigned long long*>(&P.sc->gen_over), (unsigned long long)over);
-}
-
-__global__ void k_gen_end(Params P)
-{
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        const double bm = __longlong_as_double((long long)P.sc->gen_bmax_bits);
-        if (bm > P.sc->wmax_gen) P.sc->wmax_gen = bm;
-        P.sc->gen_bmax_bits = 0ull;
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -618,7 +724,7 @@ __global__ void k_batch_begin(MultiArgs M)
     const int i = blockIdx.x;
     if (i >= M.n_inst) return;
     const Params& P = M.inst[i];
-    if (threadIdx.x == 0) begin_pass_dev(P, M.ncalls[i]);
+    begin_pass_dev(P, M.ncalls[i]);
     const size_t nd = (size_t)P.K * P.d * P.n;
     for (size_t q = threadIdx.x; q < nd; q += blockDim.x) P.D[q] = 0.0;
     for (int q = threadIdx.x; q < 2 * P.K; q += blockDim.x) P.csum[q] = 0.0;
@@ -627,10 +733,11 @@ __global__ void k_batch_begin(MultiArgs M)
         __syncthreads();
         const int64_t ncell = P.coff[P.K];
         for (int64_t q = threadIdx.x; q < ncell; q += blockDim.x) P.cellsum[q] = 0.0;
+        for (int q = threadIdx.x; q < P.K; q += blockDim.x) P.Qc[q] = 0.0;
     }
 }
 
-// Stratified instances: Q_c per (instance, channel) pair, one block each.
+// Stratified instances: Q_c per (instance, channel) pair, STRAT_PARTS blocks each.
 __global__ void k_batch_strat_q(MultiArgs M)
 {
     const int pair = blockIdx.x;
@@ -641,17 +748,17 @@ __global__ void k_batch_strat_q(MultiArgs M)
     }
     const Params& P = M.inst[lo];
     if (!P.stratified) return;
-    strat_q_channel(P, pair - M.pair_off[lo]);
+    strat_q_channel(P, pair - M.pair_off[lo], blockIdx.y, gridDim.y);
 }
 
 // Work items: every (instance, channel) pair with N_c calls gives
 // ceil(N_c / item_calls) items; exclusive prefix over the pairs.
 __global__ void k_batch_items(MultiArgs M)
 {
-    __shared__ long long part[1024];
+    __shared__ long long tmp[33];
     const int tid = threadIdx.x, nt = blockDim.x;
     const int per = (M.npairs + nt - 1) / nt;
-    const int p0 = tid * per, p1 = min(M.npairs, p0 + per);
+    const int p0 = min(M.npairs, tid * per), p1 = min(M.npairs, p0 + per);
     auto items_of = [&](int pr) -> long long {
         int lo = 0, hi = M.n_inst - 1; // instance with pair_off[i] <= pr
         while (lo < hi) {
@@ -663,17 +770,13 @@ __global__ void k_batch_items(MultiArgs M)
     };
     long long s = 0;
     for (int pr = p0; pr < p1; ++pr) s += items_of(pr);
-    part[tid] = s;
-    __syncthreads();
+    long long total;
+    long long off = block_scan(s, tmp, &total) - s;
     if (tid == 0) {
-        long long a = 0;
-        for (int q = 0; q < nt; ++q) { const long long v = part[q]; part[q] = a; a += v; }
-        M.ctl->total = a;
+        M.ctl->total = total;
         M.ctl->next = 0;
-        M.pair_prefix[M.npairs] = a;
+        M.pair_prefix[M.npairs] = total;
     }
-    __syncthreads();
-    long long off = part[tid];
     for (int pr = p0; pr < p1; ++pr) {
         M.pair_prefix[pr] = off;
         off += items_of(pr);
@@ -706,7 +809,7 @@ __global__ void __launch_bounds__(REFINE_WARPS * 32) k_batch_refine(MultiArgs M)
         const int mid = (lo + hi + 1) >> 1;
         if (M.row_off[mid] <= row) lo = mid; else hi = mid - 1;
     }
-    refine_row_dev(M.inst[lo], row - M.row_off[lo], lane, rs + (size_t)wid * (4 * M.max_n + 2));
+    refine_row_dev(M.inst[lo], row - M.row_off[lo], lane, rs + (size_t)wid * refine_scratch(M.max_n));
 }
 
 // one block per instance
@@ -730,7 +833,7 @@ cudaError_t launch_batch_after(const MultiArgs& M, cudaStream_t s)
 {
     cudaError_t e;
     if (M.any_strat) {
-        k_batch_strat_q<<<M.npairs, 256, 0, s>>>(M);
+        k_batch_strat_q<<<dim3(M.npairs, STRAT_PARTS), 256, 0, s>>>(M);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
@@ -738,7 +841,7 @@ cudaError_t launch_batch_after(const MultiArgs& M, cudaStream_t s)
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int blocks = (M.nrows + REFINE_WARPS - 1) / REFINE_WARPS;
-    k_batch_refine<<<blocks, REFINE_WARPS * 32, (size_t)REFINE_WARPS * (4 * M.max_n + 2) * sizeof(double), s>>>(M);
+    k_batch_refine<<<blocks, REFINE_WARPS * 32, (size_t)REFINE_WARPS * refine_scratch(M.max_n) * sizeof(double), s>>>(M);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_batch_alpha<<<M.n_inst, 64, 0, s>>>(M);
@@ -776,15 +879,18 @@ cudaError_t launch_wait_selftest(long long limit, unsigned int* flag, long long*
 // ---------------------------------------------------------------------------
 // host-side launchers
 // ---------------------------------------------------------------------------
-cudaError_t launch_begin_pass(const Params& P, int64_t N, cudaStream_t s)
+cudaError_t launch_begin_pass(const Params& P, int64_t N, cudaStream_t s, int clear, int64_t cells)
 {
-    k_begin_pass<<<1, 32, 0, s>>>(P, N);
+    // a block for every 4096 words to clear, up to two per SM
+    const int64_t words = clear ? (int64_t)P.K * P.d * P.n + (P.stratified ? cells : 0) : 0;
+    const int blocks = (int)std::min<int64_t>(304, std::max<int64_t>(1, words / 4096));
+    k_begin_pass<<<blocks, 256, 0, s>>>(P, N, clear, cells);
     return cudaGetLastError();
 }
 
 cudaError_t launch_strat_q(const Params& P, cudaStream_t s)
 {
-    k_strat_q<<<P.K, 256, 0, s>>>(P);
+    k_strat_q<<<dim3(P.K, STRAT_PARTS), 256, 0, s>>>(P);
     return cudaGetLastError();
 }
 
@@ -798,7 +904,7 @@ cudaError_t launch_derive(const Params& P, cudaStream_t s)
 {
     const int rows = P.K * P.d;
     const int blocks = min((rows + 3) / 4, 1024);
-    k_derive<<<blocks, 128, 0, s>>>(P);
+    k_derive<<<blocks, 128, (size_t)4 * (P.n + 1) * sizeof(int), s>>>(P);
     return cudaGetLastError();
 }
 
@@ -806,7 +912,7 @@ cudaError_t launch_refine(const Params& P, cudaStream_t s)
 {
     const int rows = P.K * P.d;
     const int blocks = (rows + REFINE_WARPS - 1) / REFINE_WARPS;
-    const size_t sm = (size_t)REFINE_WARPS * (4 * P.n + 2) * sizeof(double);
+    const size_t sm = (size_t)REFINE_WARPS * refine_scratch(P.n) * sizeof(double);
     k_refine<<<blocks, REFINE_WARPS * 32, sm, s>>>(P);
     return cudaGetLastError();
 }
@@ -825,7 +931,7 @@ cudaError_t launch_update_alpha(const Params& P, cudaStream_t s)
 
 cudaError_t launch_gen_prepare(const Params& P, cudaStream_t s)
 {
-    k_gen_prepare<<<1, 32, 0, s>>>(P);
+    k_gen_prepare<<<1, P.K > 128 ? 256 : (P.K + 31) / 32 * 32, 0, s>>>(P);
     return cudaGetLastError();
 }
 
@@ -836,9 +942,6 @@ cudaError_t launch_gen_finish(const Params& P, const PassArgs& G, int64_t remain
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_gen_copy<<<(unsigned)G.nchunks, 256, 0, s>>>(P, G, out);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_gen_end<<<1, 32, 0, s>>>(P);
     return cudaGetLastError();
 }
 

@@ -132,14 +132,12 @@ extern "C" vamp_status vamp_sample_pass_static(const vamp_config* cfg, const dou
     pr.edges64 = const_cast<double*>(dev_edges);  // read only by the kernels launched here
     pr.alpha = const_cast<double*>(dev_alpha);    // read only by the kernels launched here
     const size_t rows = (size_t)K * d;
-    // everything that must start from zero: accumulators and scalars
-    e = cudaMemsetAsync(pr.D, 0, rows * n * 8, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(pr.csum, 0, 2 * K * 8, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(pr.sc, 0, sizeof(Scalars), stream);
+    // what must start from zero: the scalars (the pass accumulators: launch_begin_pass)
+    e = cudaMemsetAsync(pr.sc, 0, sizeof(Scalars), stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(pr.shift, dev_shift, K * 8, cudaMemcpyDeviceToDevice, stream);
     if (e == cudaSuccess) e = vamp::upload_setup(pr, S, stream);
     if (e == cudaSuccess) e = vamp::launch_derive(pr, stream);
-    if (e == cudaSuccess) e = vamp::launch_begin_pass(pr, n_calls, stream);
+    if (e == cudaSuccess) e = vamp::launch_begin_pass(pr, n_calls, stream, 1);
     if (e == cudaSuccess) {
         vamp::PassArgs A{};
         A.field = iteration;

@@ -192,6 +192,7 @@ bool build_setup(const vamp_config* cfg, Params& pr, Setup& S, std::string& why)
     S.d = d; S.K = K; S.n = n; S.P = P;
     S.fp32 = cfg->precision == VAMP_PREC_FP32_EVAL;
     pr.d = d; pr.K = K; pr.n = n; pr.P = P;
+    pr.fp32 = S.fp32;
     pr.key0 = (uint32_t)(cfg->seed & 0xffffffffu);
     pr.key1 = (uint32_t)(cfg->seed >> 32);
     pr.request = cfg->request_id;

@@ -292,4 +292,21 @@ VAMP_HD Sf sf_exp2(double x)
     return Sf{sf_mulhi(v, (i & 2u) ? k23 : k01) << 1, n - 63};
 }
 
+// log2 of a positive normal double: an FP32 logarithm y0 of the significand m
+// in [1, 2), then log2 (m 2^-y0) = d - d^2/2 + ... over ln 2 with d = m 2^-y0 - 1
+// (|d| < 2^-20) from the 64-bit product.  Absolute error about 2^-59 besides
+// the rounding of the sum.
+VAMP_HD double sf_log2(double x)
+{
+    const uint64_t b = sf_bits(x);
+    const uint64_t m = (b << 11) | (1ull << 63);
+    const int ex = (int)((uint32_t)(b >> 52) & 0x7ffu) - 1023;
+    const double y0 = (double)(sf_lg2f((float)(uint32_t)(m >> 40)) - 23.0f);  // in [0, 1]
+    const Sf t = sf_exp2(-y0);
+    const Sf p = sf_mul(Sf{m, -63}, t);                               // about 1; p.e is -63 or -62
+    const int64_t d = (int64_t)((p.m << (63 + p.e)) - (1ull << 63));  // Q1.63
+    const double dd = (double)d * 0x1p-63;
+    return (y0 + (double)ex) + (dd - 0.5 * dd * dd) * 1.4426950408889634;
+}
+
 }  // namespace vamp
