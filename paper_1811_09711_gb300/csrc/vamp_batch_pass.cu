@@ -63,9 +63,8 @@ __device__ __forceinline__ bool run_item(const MultiArgs& M, const Params& P, Sm
     for (int64_t bt = 0; bt < nb; ++bt) {
         const int64_t base = a + bt * B, end = min(b, base + B);
         Calls<T, CPT, SH::DM> C;
-        phase_a<T, 0, CPT>(P, sh, M.iter[inst], base, end, c, C);
         SoftCall<SH::DM> soft;
-        if constexpr (sizeof(T) == 8) soft_prepare(P, sh, C.p[0], C.Aexp[0], soft);
+        phase_a<T, 0, CPT>(P, sh, M.iter[inst], base, end, c, C, &soft);
         for (int t = 0; t < ntiles; ++t) {
             const int bb = streaming ? (int)(u & 1) : t;
             if (streaming || bt == 0) {

@@ -89,6 +89,7 @@ struct alignas(16) ChanHdr<double> {
     uint32_t bw;         // some are Breit-Wigner
     uint8_t sk[MAXMAP];  // their coordinate | kind << 4
     double c0[MAXMAP], c1[MAXMAP];    // Breit-Wigner: m, Γ²; power law: δ
+    double fw[MAXMAP][3];             // Breit-Wigner: Γ, A, atan(m/Γ)
     float pinvG[MAXMAP], pt0[MAXMAP], pscale[MAXMAP];  // FP32 inverse map to cells: (atan(dp/Γ) + t0) scale; x scale
     double sp[MAXMAP][SP_N];  // per slot: m, Γ, A, Γ², 1/Γ, Γ/A, 1/A, atan(m/Γ), δ, 1/powN
 };
@@ -247,7 +248,7 @@ template <> struct Prec<double> {
     static __device__ __forceinline__ double gcen(const Params& P) { return P.gcen; }
     static __device__ __forceinline__ double gk2(const Params& P) { return P.gk2; }
     // in-bin fraction of the forward map: the exact 33-bit value
-    static __device__ __forceinline__ double frac(uint64_t low33) { return (double)low33 * 0x1p-33; }
+    static __device__ __forceinline__ double frac(uint64_t low33) { return sf_frac33(low33); }
     // in-bin fraction of a stratified call: remainder over n_r 2^33, one
     // correctly rounded division
     static __device__ __forceinline__ double frac_div(uint64_t rem, uint64_t den)
@@ -259,7 +260,7 @@ template <> struct Prec<double> {
     {
         return __dadd_rn(e0, __dmul_rn(fr, __dsub_rn(e1, e0)));
     }
-    static __device__ __forceinline__ double tan_(double v) { return tan(v); }
+    static __device__ __forceinline__ double tan_(double v) { return sf_tan(v); }
     static __device__ __forceinline__ double atan_(double v) { return atan(v); }
     // v^(-1/5) for a normal v > 0 (Newton's method for the inverse fifth
     // root): with v = m 2^E, m in [1, 2), write -E = 5a + r (r in 0..4), so
@@ -466,7 +467,7 @@ __device__ __forceinline__ int lookup(const SH& sh, const unsigned char* row, in
 // ---------------------------------------------------------------------------
 // Forward map of the selected channel (lookup block in global memory):
 // r -> x_c -> p, the own term g_c(x_c)/φ'_c(x_c) and the Gaussian exponent
-// sum of p (log2 units).
+// sum of p (log2 units).  FP32; the FP64 form is soft_forward.
 // ---------------------------------------------------------------------------
 template <typename T, class SH>
 __device__ __forceinline__ void forward_call(const Params& P, const SH& sh, int c, const uint32_t* X,
@@ -495,17 +496,10 @@ __device__ __forceinline__ void forward_call(const Params& P, const SH& sh, int 
                 fr = Prec<T>::frac(t & ((1ull << 33) - 1ull));
             }
             const unsigned char* row = sh.row(blk, k);
-            // the grid's edges: the FP32 block row, or the FP64 master grid
-            // (whose values the FP64 block holds only for unmapped rows)
-            const T* e = sizeof(T) == 8
-                             ? reinterpret_cast<const T*>(P.edges64 + ((size_t)c * d + k) * (size_t)(n + 1))
-                             : reinterpret_cast<const T*>(row);
+            const T* e = reinterpret_cast<const T*>(row);
             x[k] = Prec<T>::lerp(__ldg(e + j), __ldg(e + j + 1), fr);
             jf[k] = j;
-            if constexpr (sizeof(T) == 8)
-                g *= sf_unpack_double(__ldg(reinterpret_cast<const unsigned long long*>(row + sh.dens_off()) + j));
-            else
-                g *= __ldg(reinterpret_cast<const T*>(row + sh.dens_off()) + j);
+            g *= __ldg(reinterpret_cast<const T*>(row + sh.dens_off()) + j);
         } else {
             x[k] = T(0);
             jf[k] = 0;
@@ -679,36 +673,110 @@ struct SoftCall {
     double A;  // Σ a_k
 };
 
-template <class SH>
-__device__ __forceinline__ void soft_prepare(const Params& P, const SH& sh, const double (&p)[SH::DM], double A,
-                                             SoftCall<SH::DM>& S)
-{
-#pragma unroll
-    for (int k = 0; k < SH::DM; ++k) {
-        if (sh.has(k)) {
-            S.q[k] = Prec<double>::cell(p[k], sh.lshift());
-            S.p[k] = p[k];
-        }
-    }
-    for (uint32_t m = P.map_any; m; m &= m - 1u) {
-        const int k = __ffs(m) - 1;
-        const double pk = S.p[k];
-        if (P.matching) {
-            const double u = pk - P.gcen;
-            const double a = u * u * P.gk2;
-            S.E[k] = P.gauss_sum ? sf_bits(a) : sf_pack(sf_exp2(a));
-        }
-        if ((P.pow_any >> k) & 1u) S.W[k] = sf_pack(sf_powm08(pk));
-    }
-    S.A = A;
-    S.e0 = P.matching && !P.gauss_sum ? sf_exp2(-A) : Sf{1ull << 63, -63};
-}
-
 // One packed factor onto acc; the exponents' biases are added by the caller.
 __device__ __forceinline__ void soft_factor(uint64_t& acc, int& ae, uint64_t w)
 {
     acc = sf_mulhi(acc, w & ~2047ull);
     ae += (int)((uint32_t)w & 2047u);
+}
+
+// Forward map of a call of channel c (lookup block and master grid in global
+// memory) and what the channel loop needs of it: p, the forward bins jf, the
+// own term g_c/φ'_c without the constant gN, and S.  An FP64 operation stands
+// only where a coordinate's value is formed: the fraction, the edges'
+// interpolation, (p - centre)² and the map's ends; the tangent, the densities
+// and the own Jacobian (its denominators, and the p^(-4/5) that the channels
+// share) are on the integer pipe.  With FP64 throughout, a d = 8 call of six
+// channels kept the FP64 pipe busy for 250 operations, half of them here, and
+// the pass (1e6 calls) took 482 us.
+// digit (stratified calls, else null): the cell's base-n_r digits.  x_out (may
+// be null) receives x.
+template <class SH>
+__device__ __forceinline__ void soft_forward(const Params& P, const SH& sh, int c, const uint32_t* X,
+                                             double (&p)[SH::DM], int (&jf)[SH::DM], double& own,
+                                             SoftCall<SH::DM>& S, const uint32_t* digit = nullptr, uint32_t nr = 1u,
+                                             double* x_out = nullptr)
+{
+    const int d = sh.d(), n = sh.n();
+    const unsigned char* blk = P.lk64 + (size_t)c * sh.bytes();
+    const ChanHdr<double>* h = reinterpret_cast<const ChanHdr<double>*>(blk);
+    const double* e0 = P.edges64 + (size_t)c * d * (size_t)(n + 1);
+    uint64_t acc = 1ull << 63;
+    int ae = 0;  // acc 2^(ae - 1022 d - 63)
+#pragma unroll
+    for (int k = 0; k < SH::DM; ++k) {
+        jf[k] = 0;
+        if (sh.has(k)) {
+            double fr;
+            if (digit) {
+                // stratified call: r_k = (a_k + u_k) / n_r, from the integer
+                // (2^33 a_k + 2X + 1) n over n_r 2^33 (n_r = 1: the line below)
+                const uint64_t den = (uint64_t)nr << 33;
+                const uint64_t t = (((uint64_t)digit[k] << 33) + 2ull * X[k] + 1ull) * (uint64_t)n;
+                const uint64_t jj = t / den;
+                jf[k] = (int)jj;
+                fr = Prec<double>::frac_div(t - jj * den, den);
+            } else {
+                const uint64_t t = (2ull * X[k] + 1ull) * (uint64_t)n;
+                jf[k] = (int)(t >> 33);
+                fr = sf_frac33(t & ((1ull << 33) - 1ull));
+            }
+            const double* e = e0 + (size_t)k * (n + 1) + jf[k];
+            S.p[k] = Prec<double>::lerp(__ldg(e), __ldg(e + 1), fr);
+            if (x_out) x_out[k] = S.p[k];
+            soft_factor(acc, ae, __ldg(reinterpret_cast<const unsigned long long*>(sh.row(blk, k) + sh.dens_off()) + jf[k]));
+        }
+        if (k % 8 == 7 || k == SH::DM - 1) sf_norm(acc, ae);
+    }
+    const Sf one{1ull << 63, -63};
+    Sf den = one, G = one;
+    const int ns = (int)__ldg(&h->nslot);
+#pragma unroll 1
+    for (int s = 0; s < ns; ++s) {
+        const int w = __ldg(&h->sk[s]), k = w & 15;
+        const double x = S.p[k];
+        if ((w >> 4) == MAP_BW) {
+            const double* sp = h->fw[s];
+            const double t = __ldg(sp) * Prec<double>::tan_(__ldg(sp + 1) * x - __ldg(sp + 2));  // p - m, before p is rounded
+            const double pk = __ldg(&h->c0[s]) + t, dp = pk - __ldg(&h->c0[s]);
+            den = sf_mul(den, sf_from_double(dp * dp + __ldg(&h->c1[s])));
+            S.p[k] = pk;
+        } else {
+            const double x2 = x * x, x4 = x2 * x2;
+            double pk = x4 * x;
+            if (pk < Prec<double>::tiny()) pk = Prec<double>::tiny();
+            G = sf_mul(G, sf_rcp(sf_from_double(x4)));  // (p^(-4/5) from x: p may have been floored)
+            S.p[k] = pk;
+        }
+    }
+    const Sf y = sf_rcp(sf_norm(den));
+    own = sf_to_double(sf_norm(sf_mul(sf_mul(Sf{acc, ae - 1022 * d - 63}, sf_norm(G)), y)));
+    // Gaussian exponents, cells, and the factors of the coordinates that some
+    // channel maps
+    const double gc = P.gcen, k2 = P.gk2;
+    double A = 0.0;
+#pragma unroll
+    for (int k = 0; k < SH::DM; ++k) {
+        p[k] = 0.0;
+        if (sh.has(k)) {
+            p[k] = S.p[k];
+            S.q[k] = Prec<double>::cell(p[k], sh.lshift());
+            const double u = p[k] - gc;
+            A = fma(u, u, A);
+        }
+    }
+    A *= k2;
+    for (uint32_t m = P.map_any; m; m &= m - 1u) {
+        const int k = __ffs(m) - 1;
+        const double pk = S.p[k];
+        if (P.matching) {
+            const double u = pk - gc, a = u * u * k2;
+            S.E[k] = P.gauss_sum ? sf_bits(a) : sf_pack(sf_exp2(a));
+        }
+        if ((P.pow_any >> k) & 1u) S.W[k] = sf_pack(sf_powm08(pk));
+    }
+    S.A = A;
+    S.e0 = P.matching && !P.gauss_sum ? sf_exp2(-A) : one;
 }
 
 // Largest j' in [j, n] with e[j'] <= x, for e[j] <= x: three edges at a time,

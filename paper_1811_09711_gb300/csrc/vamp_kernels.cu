@@ -665,26 +665,31 @@ __global__ void k_eval(Params P, EvalArgs A)
             if (k == d) xc = X[k];
         c = choose_channel(P, unif64(xc));
     }
-    T x[DMAX], p1[1][DMAX], g[1], f[1], Aq[1];
+    T p1[1][DMAX], x[DMAX], g[1], f[1], Aq[1];
     int jf[DMAX];
-    T owngJ;
-    if (A.mode == 0 && P.stratified) {
-        const uint32_t nr = (uint32_t)P.nr[c];
+    uint32_t dig[DMAX], nr = 1u;
+    const bool strat = A.mode == 0 && P.stratified;
+    if (strat) {
+        nr = (uint32_t)P.nr[c];
         uint32_t cell = (uint32_t)(((int64_t)call - P.Pc[c]) / P.spc[c]);
-        uint32_t dig[DMAX];
         for (int k = 0; k < DMAX; ++k) {
             dig[k] = cell % nr;
             cell /= nr;
         }
-        forward_call<T>(P, sh, c, X, x, p1[0], jf, owngJ, Aq[0], dig, nr);
-    } else {
-        forward_call<T>(P, sh, c, X, x, p1[0], jf, owngJ, Aq[0]);
     }
-    g[0] = Prec<T>::alpha(P, c) * owngJ;
+    SoftCall<DMAX> soft;
+    if constexpr (sizeof(T) == 8) {
+        double own;
+        soft_forward(P, sh, c, X, p1[0], jf, own, soft, strat ? dig : nullptr, nr, x);
+        Aq[0] = soft.A;
+        g[0] = P.alphaN[c] * own;
+    } else {
+        T owngJ;
+        forward_call<T>(P, sh, c, X, x, p1[0], jf, owngJ, Aq[0], strat ? dig : nullptr, nr);
+        g[0] = Prec<T>::alpha(P, c) * owngJ;
+    }
     f[0] = P.matching ? T(0) : integrand_peaks<T, DMAX>(P, d, p1[0], Aq[0]);
     int* bins = A.bins + (size_t)q * P.K * d;
-    SoftCall<DMAX> soft;
-    if constexpr (sizeof(T) == 8) soft_prepare(P, sh, p1[0], Aq[0], soft);
     for (int c2 = 0; c2 < P.K; ++c2) {
         const T a = Prec<T>::alpha(P, c2);
         const bool lookups = a != T(0) && c2 != c;

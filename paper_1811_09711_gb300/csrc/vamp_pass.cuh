@@ -35,7 +35,6 @@ __device__ __forceinline__ double warp_max(double v)
     return v;
 }
 
-static_assert(PASS_THREADS == PASS_THREADS_DEV, "device copy of the CTA size");
 
 struct SmemHead {
     uint64_t bar[2];
@@ -81,13 +80,36 @@ __device__ __forceinline__ int call_of(int q)
     return warp_first<CPT>() + q * 32 + (int)(threadIdx.x & 31);
 }
 
+// f / g, 0 where g is not positive.  FP64: by the integer reciprocal, the FP64
+// division (ten operations of that pipe) where g is not a normal number or f
+// not finite.
+__device__ __forceinline__ double call_weight(float f, float g) { return g > 0.f ? (double)(f / g) : 0.0; }
+__device__ __forceinline__ double call_weight(double f, double g)
+{
+    const uint64_t b = sf_bits(g), a = sf_bits(f) & 0x7fffffffffffffffull;
+    if (b - 0x0010000000000000ull < 0x7fe0000000000000ull && a < 0x7ff0000000000000ull) return sf_div(f, g);
+    return g > 0.0 ? f / g : 0.0;
+}
+
+// The larger of wm >= 0 and |w|, and whether w is finite, from the bits (an FP64
+// compare takes the pipe that the sums need).
+__device__ __forceinline__ double max_abs(double wm, double w)
+{
+    const long long a = __double_as_longlong(wm), b = __double_as_longlong(w) & 0x7fffffffffffffffll;
+    return __longlong_as_double(a > b ? a : b);
+}
+__device__ __forceinline__ bool finite_bits(double w)
+{
+    return ((unsigned)__double2hiint(w) & 0x7ff00000u) != 0x7ff00000u;
+}
+
 // Phase A: Philox words, channel, forward map on the channel's grid, own
 // term of g(p), Gaussian exponent sum; the integrand when peaks are not the
 // channels' maps.  Call q of this thread is base + call_of(q) (integration)
 // or base + q*PASS_THREADS + tid (generation, whose records are in that order).
 template <typename T, int MODE, int CPT, class SH>
 __device__ __forceinline__ void phase_a(const Params& P, const SH& sh, uint32_t field, int64_t base, int64_t end,
-                                        int cseg, Calls<T, CPT, SH::DM>& C)
+                                        int cseg, Calls<T, CPT, SH::DM>& C, SoftCall<SH::DM>* soft = nullptr)
 {
     constexpr int DM = SH::DM;
     const int d = sh.d();
@@ -113,24 +135,32 @@ __device__ __forceinline__ void phase_a(const Params& P, const SH& sh, uint32_t 
             C.xacc[q] = xa;
         }
         C.cq[q] = c;
-        T x[DM];
         int jf[DM];
-        T owngJ, Aq;
-        if (MODE == 0 && SH::kStrat && P.stratified) {
+        uint32_t dig[DM], nr = 1u;
+        const bool strat = MODE == 0 && SH::kStrat && P.stratified;
+        if (strat) {
             // cell of the call and its base-n_r digits (§3.3)
-            const uint32_t nr = (uint32_t)P.nr[c];
+            nr = (uint32_t)P.nr[c];
             uint32_t cell = (uint32_t)(((C.valid[q] ? i : base) - P.Pc[c]) / P.spc[c]);
-            uint32_t dig[DM];
 #pragma unroll
             for (int k = 0; k < DM; ++k) {
                 dig[k] = cell % nr;
                 cell /= nr;
             }
-            forward_call<T>(P, sh, c, X, x, C.p[q], jf, owngJ, Aq, dig, nr);
-        } else {
-            forward_call<T>(P, sh, c, X, x, C.p[q], jf, owngJ, Aq);
         }
-        C.Aexp[q] = Aq;
+        if constexpr (sizeof(T) == 8) {
+            double own;
+            if (strat) soft_forward(P, sh, c, X, C.p[q], jf, own, *soft, dig, nr);
+            else soft_forward(P, sh, c, X, C.p[q], jf, own, *soft);
+            C.Aexp[q] = soft->A;
+            C.g[q] = __ldg(P.alphaN + c) * own;
+        } else {
+            T x[DM], owngJ, Aq;
+            if (strat) forward_call<T>(P, sh, c, X, x, C.p[q], jf, owngJ, Aq, dig, nr);
+            else forward_call<T>(P, sh, c, X, x, C.p[q], jf, owngJ, Aq);
+            C.Aexp[q] = Aq;
+            C.g[q] = Prec<T>::alpha(P, c) * owngJ;
+        }
 #pragma unroll
         for (int w = 0; w < (DM + 3) / 4; ++w) {
             uint32_t v = 0;
@@ -139,8 +169,7 @@ __device__ __forceinline__ void phase_a(const Params& P, const SH& sh, uint32_t 
                 if (4 * w + b < DM) v |= (uint32_t)(jf[4 * w + b] & 0xff) << (8 * b);
             C.jp[q][w] = v;
         }
-        C.g[q] = Prec<T>::alpha(P, c) * owngJ;
-        C.f[q] = P.matching ? T(0) : integrand_peaks<T, DM>(P, d, C.p[q], Aq);
+        C.f[q] = P.matching ? T(0) : integrand_peaks<T, DM>(P, d, C.p[q], C.Aexp[q]);
     }
 }
 
@@ -202,14 +231,14 @@ __device__ __forceinline__ void phase_c_int(const SH& sh, const Calls<T, CPT, SH
 #pragma unroll
     for (int q = 0; q < CPT; ++q) {
         if (!C.valid[q]) continue;
-        double w = C.g[q] > T(0) ? (double)(C.f[q] / C.g[q]) : 0.0;
-        if (!isfinite(w)) { bad = true; w = 0.0; }
+        double w = call_weight(C.f[q], C.g[q]);
+        if (!finite_bits(w)) { bad = true; w = 0.0; }
         const double dv = w - sft;
         s1 += dv;
         s2 += dv * dv;
         if (cs.sum)  // stratified: the sum of the call's cell
             atomicAdd(&cs.sum[cs.coff + (cs.l0 + call_of<CPT>(q)) / cs.spc], dv);
-        wm = fmax(wm, fabs(w));  // signed integrands: w_max bounds |w|
+        wm = max_abs(wm, w);  // signed integrands: w_max bounds |w|
         const double w2 = w * w;
 #pragma unroll
         for (int s = 0; s < DM; ++s) {
@@ -247,9 +276,9 @@ __device__ __forceinline__ void phase_c_gen(const Params& P, const PassArgs& A, 
         double w = 0.0;
         bool acc = false;
         if (C.valid[q]) {
-            w = C.g[q] > T(0) ? (double)(C.f[q] / C.g[q]) : 0.0;
-            if (!isfinite(w)) { bad = true; w = 0.0; }
-            wm = fmax(wm, fabs(w));
+            w = call_weight(C.f[q], C.g[q]);
+            if (!finite_bits(w)) { bad = true; w = 0.0; }
+            wm = max_abs(wm, w);
             acc = unif64(C.xacc[q]) * wmax < fabs(w);  // the event keeps the sign of w
         }
         const unsigned bal = __ballot_sync(0xffffffffu, acc);
@@ -416,11 +445,7 @@ __device__ __forceinline__ void pass_body(const Params& P, const PassArgs& A)
         // ---- phase A: own channel forward map, integrand --------------------
         Calls<T, CPT, DM> C;
         const bool live = MODE == 1 || base + warp_first<CPT>() < end;  // some call of this warp
-        if (live) phase_a<T, MODE, CPT>(P, sh, A.field, base, end, cseg, C);
-        if constexpr (sizeof(T) == 8) {
-            static_assert(CPT == 1, "the FP64 channel loop takes one call per thread");
-            if (live) soft_prepare(P, sh, C.p[0], C.Aexp[0], soft);
-        }
+        if (live) phase_a<T, MODE, CPT>(P, sh, A.field, base, end, cseg, C, &soft);
 
         // ---- phase B: every channel's term of g(p) (and the matching peaks) --
         for (int t = 0; t < ntiles; ++t) {

@@ -131,6 +131,9 @@ void make_hdr(const vamp_map_desc& r, double weight, double zinv, int d, int lsh
                 h.bw = 1;
                 h.c0[q] = h.sp[s][SP_M];
                 h.c1[q] = h.sp[s][SP_G2];
+                h.fw[q][0] = h.sp[s][SP_G];
+                h.fw[q][1] = A;
+                h.fw[q][2] = h.sp[s][SP_T0];
                 h.gN *= h.sp[s][SP_GINVA];
                 h.fN *= h.sp[s][SP_GINVA];
                 if (!(h.sp[s][SP_G2] >= 2.3e-308)) h.gN = h.fN = NAN;  // Γ² vanishes

@@ -309,4 +309,58 @@ VAMP_HD double sf_log2(double x)
     return (y0 + (double)ex) + (dd - 0.5 * dd * dd) * 1.4426950408889634;
 }
 
+// tan of a double |th| < pi/2, to about 2^-58: the ninth convergent of Lambert's
+// continued fraction, tan z = z N(z^2) / D(z^2) within 6e-19 for z <= pi/4, with
+// tan = D / (z N) of z = pi/2 - |th| above.  N and D are taken in 64-bit fixed
+// point (each inner sum is positive), z with its own exponent.
+VAMP_HD double sf_tan(double th)
+{
+    const uint64_t b = sf_bits(th) & 0x7fffffffffffffffull;
+    const bool far = b >= 0x3fe921fb54442d18ull;  // above pi/4
+    Sf z = sf_from_double(sf_from_bits(b));
+    if (b < 0x0010000000000000ull) return th;
+    if (far) {
+        // pi/2 - |th| (whose 53 bits lie above 2^-63) in Q1.63 and 64 bits more
+        uint64_t m = 0xc90fdaa22168c234ull - (z.m >> (-63 - z.e)), lo = 0xc4c6628b80dc1cd1ull;
+        int e = -63;
+        if (!(m >> 32)) { m = (m << 32) | (lo >> 32); lo <<= 32; e -= 32; }
+        if (!(m >> 32)) { m = (m << 32) | (lo >> 32); lo <<= 32; e -= 32; }
+#ifdef __CUDA_ARCH__
+        const int s = __clz((int)(m >> 32)) & 31;
+#else
+        const int s = __builtin_clz((uint32_t)(m >> 32) | 1u) & 31;
+#endif
+        m = (m << s) | (uint64_t)((uint32_t)(lo >> 32) >> 1 >> (31 - s));
+        e -= s;
+        z = Sf{m, e};
+    }
+    const int sh = -64 - z.e;  // z < 1
+    const uint64_t q = sh < 64 ? z.m >> sh : 0ull, v = sf_mulhi(q, q);  // z^2, Q0.64
+    uint64_t N = 0x1e20001e20002ull - sf_mulhi(v, 0x7ca36d9c30ull);
+    N = 0x101010101010101ull - sf_mulhi(v, N);
+    N = 0x2323232323232323ull - sf_mulhi(v, N);
+    N = ~sf_mulhi(v, N);  // 1 - ..., Q0.64 (short of it by 2^-64)
+    uint64_t d = 0x1a5c001a5c001aull - sf_mulhi(v, 0x15e8ba44745dull);
+    d = 0x707070707070707ull - sf_mulhi(v, d);
+    d = 0x7878787878787878ull - sf_mulhi(v, d);
+    d = ~sf_mulhi(v, d);
+    const Sf zn = sf_mul(z, Sf{N, -64}), dd{d, -64};
+    const Sf t = far ? sf_mul(dd, sf_rcp(sf_norm(zn))) : sf_mul(zn, sf_rcp(sf_norm(dd)));
+    const double r = sf_to_double(sf_norm(t));
+    return sf_bits(th) >> 63 ? -r : r;
+}
+
+// a / b of doubles, b > 0 normal and a / b not below the normal range, to about
+// 2^-53: the reciprocal above (0 / b = 0).
+VAMP_HD double sf_div(double a, double b)
+{
+    const uint64_t ua = sf_bits(a);
+    if ((ua << 1) < (1ull << 53)) return a * 0.0;  // zero or subnormal
+    const double q = sf_to_double(sf_norm(sf_mul(sf_from_double(a), sf_rcp(sf_from_double(b)))));
+    return ua >> 63 ? -q : q;
+}
+
+// n 2^-33 of a 33-bit integer, exact: the fraction of 1.xxx less 1.
+VAMP_HD double sf_frac33(uint64_t n) { return sf_from_bits(0x3ff0000000000000ull | (n << 19)) - 1.0; }
+
 }  // namespace vamp

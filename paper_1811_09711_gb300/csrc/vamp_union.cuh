@@ -337,11 +337,11 @@ __global__ void __launch_bounds__(PASS_THREADS, MINB) k_union(Params P, PassArgs
             // the warp's shifted sums go out once per batch
             if (C.valid[0]) {
                 double w = C.g[0] > 0.f ? (double)(C.f[0] / C.g[0]) : 0.0;
-                if (!isfinite(w)) { bad = true; w = 0.0; }
+                if (!finite_bits(w)) { bad = true; w = 0.0; }
                 const double dv = w - sft;
                 s1 = dv;
                 s2 = dv * dv;
-                wm = fmax(wm, fabs(w));  // signed integrands: w_max bounds |w|
+                wm = max_abs(wm, w);  // signed integrands: w_max bounds |w|
                 const double w2 = w * w;
                 double* Dc = P.D + (size_t)cseg * dn;
 #pragma unroll
