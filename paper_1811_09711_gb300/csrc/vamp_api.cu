@@ -246,7 +246,8 @@ vamp_status choose_variant(vamp_ctx* c, int64_t n_calls)
         if (it != g_tuned.end()) best = it->second;
     }
     if (best && std::find(cand.begin(), cand.end(), best) == cand.end()) best = nullptr;  // not a candidate here
-    if (!best && cand.size() == 1) best = cand[0];
+    // FP64: the kernel of the range of d was the faster one at every size measured
+    if (!best && (cand.size() == 1 || !c->fp32)) best = cand[0];
     if (!best) {
         // time each candidate on a pass of `probe` calls over the current
         // grids; the pass result is discarded (no finish kernel runs) and

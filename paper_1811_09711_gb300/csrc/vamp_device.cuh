@@ -761,19 +761,19 @@ __device__ __forceinline__ void soft_forward(const Params& P, const SH& sh, int 
         if (sh.has(k)) {
             p[k] = S.p[k];
             S.q[k] = Prec<double>::cell(p[k], sh.lshift());
-            const double u = p[k] - gc;
-            A = fma(u, u, A);
+            const double u = p[k] - gc, u2 = u * u;
+            A += u2;
+            if ((P.map_any >> k) & 1u) S.E[k] = sf_bits(u2);
         }
     }
     A *= k2;
     for (uint32_t m = P.map_any; m; m &= m - 1u) {
         const int k = __ffs(m) - 1;
-        const double pk = S.p[k];
         if (P.matching) {
-            const double u = pk - gc, a = u * u * k2;
+            const double a = sf_from_bits(S.E[k]) * k2;
             S.E[k] = P.gauss_sum ? sf_bits(a) : sf_pack(sf_exp2(a));
         }
-        if ((P.pow_any >> k) & 1u) S.W[k] = sf_pack(sf_powm08(pk));
+        if ((P.pow_any >> k) & 1u) S.W[k] = sf_pack(sf_powm08(S.p[k]));
     }
     S.A = A;
     S.e0 = P.matching && !P.gauss_sum ? sf_exp2(-A) : one;

@@ -376,7 +376,8 @@ __device__ __forceinline__ void pass_body(const Params& P, const PassArgs& A)
         // whole warps of calls, so that a small pass has few half-empty ones
         r0 = (N * blockIdx.x / gridDim.x) & ~int64_t(31);
         r1 = blockIdx.x + 1 < gridDim.x ? (N * (blockIdx.x + 1) / gridDim.x) & ~int64_t(31) : N;
-        if (r1 - r0 < (int64_t)n << dshift) dshift = 0;  // fewer d-value adds than words to clear and sum
+        // copies only as far as the calls outnumber the words to clear and sum
+        while (dshift > 0 && r1 - r0 < (int64_t)(4 * n) << dshift) --dshift;
         int64_t i = r0;
         while (i < r1) {
             const int c = find_channel(P.Pc, K, i);

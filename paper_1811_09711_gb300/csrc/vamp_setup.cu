@@ -360,7 +360,7 @@ cudaError_t upload_setup(const Params& P, const Setup& S, cudaStream_t s)
 // 32-problem batch lost more than they gained (8.65 -> 9.99 ms).
 TilePlan plan_tiles(size_t S, int K, int dn, size_t fixed, size_t budget)
 {
-    const size_t most = 8 * 1024, one = (size_t)dn * 8;
+    const size_t most = 16 * 1024, one = (size_t)dn * 8;
     int ds = 5;
     while (ds > 0 && ((one << ds) > most || fixed + 2 * S + (one << ds) > budget)) --ds;
     const size_t d = one << ds;
@@ -412,6 +412,10 @@ std::vector<const PassVariant*> pass_candidates(int fp32, int d, int n, int stra
         if (v.D == d && v.NB == n && !stratified) exact.push_back(&v);
         else if (v.D == 0 && v.NB == 0 && (stratified ? v.dhi == 0 : v.dlo <= d && d <= v.dhi)) generic.push_back(&v);
     }
+    // FP64: the any-shape form stays selectable behind the kernel of the range
+    if (!fp32 && !stratified)
+        for (const PassVariant& v : all)
+            if (!v.fp32 && v.D == 0 && v.NB == 0 && v.dhi == 0) generic.push_back(&v);
     for (const PassVariant* v : generic) exact.push_back(v);
     for (const PassVariant* v : uexact) exact.push_back(v);
     for (const PassVariant* v : ugeneric) exact.push_back(v);
