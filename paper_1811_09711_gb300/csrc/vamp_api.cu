@@ -44,7 +44,12 @@ struct vamp_ctx {
     int have_pass = 0;
     Params prm{};
     void* arena = nullptr;
-    Scalars* h_head = nullptr;   // pinned copy of the Scalars head
+    // pinned staging: [edges, where they are small][α][shifts][Scalars head],
+    // laid out as the arena's first range, so that the state moves in one copy
+    unsigned char* h_stage = nullptr;
+    size_t stage_lo = 0;         // arena offset that h_stage starts at
+    vamp::Arena ar{};
+    Scalars* h_head = nullptr;   // its Scalars head
     // generation staging (allocated on first use)
     unsigned char* g_staging = nullptr;
     uint32_t* g_callidx = nullptr;
@@ -64,6 +69,10 @@ struct vamp_ctx {
 
 namespace {
 
+// Grids up to this size go through the pinned staging buffer (a copy to or
+// from the caller's pageable memory costs about 10 us more than one from
+// there; beyond it the host's own copying does); larger ones directly.
+constexpr size_t STAGED_EDGES = 64 * 1024;
 constexpr size_t HEAD_BYTES = offsetof(Scalars, n_hist) + sizeof(int32_t) * 2;
 
 vamp_status fail(vamp_ctx* c, vamp_status s, const std::string& msg)
@@ -335,7 +344,7 @@ void vamp_destroy(vamp_ctx* c)
         cudaFree(c->g_callidx);
         cudaFree(c->g_counts);
         cudaFree(c->g_offsets);
-        cudaFreeHost(c->h_head);
+        cudaFreeHost(c->h_stage);
         if (c->ev[0]) cudaEventDestroy(c->ev[0]);
         if (c->ev[1]) cudaEventDestroy(c->ev[1]);
         for (auto& pr : c->prof_pending) { cudaEventDestroy(pr.first); cudaEventDestroy(pr.second); }
@@ -365,8 +374,11 @@ vamp_status vamp_create(const vamp_config* cfg, void* cuda_stream, vamp_ctx** ou
     DeviceGuard g(c->dev);
     cudaError_t e = cudaMalloc(&c->arena, ar.bytes);
     if (e != cudaSuccess) { delete c; return e == cudaErrorMemoryAllocation ? VAMP_ERR_OOM : VAMP_ERR_CUDA; }
-    e = cudaMallocHost((void**)&c->h_head, sizeof(Scalars));
+    c->ar = ar;
+    c->stage_lo = ar.alpha - ar.edges64 <= STAGED_EDGES ? ar.edges64 : ar.alpha;
+    e = cudaMallocHost((void**)&c->h_stage, ar.sc + HEAD_BYTES - c->stage_lo);
     if (e != cudaSuccess) { vamp_destroy(c); return VAMP_ERR_OOM; }
+    c->h_head = reinterpret_cast<Scalars*>(c->h_stage + (ar.sc - c->stage_lo));
     vamp::bind_arena(pr, (unsigned char*)c->arena, ar);
     c->prm = pr;
     Params& P = c->prm;
@@ -386,7 +398,7 @@ vamp_status vamp_create(const vamp_config* cfg, void* cuda_stream, vamp_ctx** ou
     CREATE_CK(cudaMemsetAsync(c->arena, 0, ar.bytes, c->stream));
     CREATE_CK(cudaMemcpyAsync(P.edges64, edges.data(), edges.size() * 8, cudaMemcpyHostToDevice, c->stream));
     CREATE_CK(cudaMemcpyAsync(P.alpha, alpha.data(), K * 8, cudaMemcpyHostToDevice, c->stream));
-    CREATE_CK(vamp::upload_setup(P, S, c->stream));
+    CREATE_CK(vamp::upload_setup(P, S, c->stream, true));
     CREATE_CK(vamp::launch_derive(P, c->stream));
     CREATE_CK(cudaStreamSynchronize(c->stream));
     {
@@ -606,19 +618,57 @@ vamp_status vamp_get_state(vamp_ctx* c, double* edges, double* alpha, double* sh
 {
     if (!c) return VAMP_ERR_INVALID_ARG;
     DeviceGuard g(c->dev);
-    const size_t rows = (size_t)c->K * c->d;
-    if (edges) VAMP_CK(c, cudaMemcpyAsync(edges, c->prm.edges64, rows * (c->n + 1) * 8, cudaMemcpyDeviceToHost, c->stream));
-    if (alpha) VAMP_CK(c, cudaMemcpyAsync(alpha, c->prm.alpha, c->K * 8, cudaMemcpyDeviceToHost, c->stream));
-    if (shift) VAMP_CK(c, cudaMemcpyAsync(shift, c->prm.shift, c->K * 8, cudaMemcpyDeviceToHost, c->stream));
-    vamp_status s = read_head(c);
-    if (s != VAMP_OK) return s;
+    const size_t eb = (size_t)c->K * c->d * (c->n + 1) * 8, lo = c->stage_lo;
+    const bool staged = lo == c->ar.edges64;
+    if (edges && !staged)
+        VAMP_CK(c, cudaMemcpyAsync(edges, c->prm.edges64, eb, cudaMemcpyDeviceToHost, c->stream));
+    VAMP_CK(c, cudaMemcpyAsync(c->h_stage, (unsigned char*)c->arena + lo, c->ar.sc + HEAD_BYTES - lo,
+                               cudaMemcpyDeviceToHost, c->stream));
+    VAMP_CK(c, cudaStreamSynchronize(c->stream));
+    if (edges && staged) std::memcpy(edges, c->h_stage, eb);
+    if (alpha) std::memcpy(alpha, c->h_stage + (c->ar.alpha - lo), (size_t)c->K * 8);
+    if (shift) std::memcpy(shift, c->h_stage + (c->ar.shift - lo), (size_t)c->K * 8);
     if (w_max) *w_max = c->h_head->wmax_gen;
     return VAMP_OK;
 }
 
-vamp_status vamp_set_state(vamp_ctx* c, const double* edges, const double* alpha, const double* shift, double w_max)
+namespace {
+
+// State from host arrays (null: kept), already validated; n_hist >= 0: also
+// the length of the history of passes.
+vamp_status upload_state(vamp_ctx* c, const double* edges, const double* alpha, const double* shift, double w_max,
+                         int n_hist)
 {
-    if (!c) return VAMP_ERR_INVALID_ARG;
+    DeviceGuard g(c->dev);
+    const size_t eb = (size_t)c->K * c->d * (c->n + 1) * 8, kb = (size_t)c->K * 8, lo = c->stage_lo;
+    const bool staged = lo == c->ar.edges64;
+    unsigned char* base = (unsigned char*)c->arena;
+    if (edges && staged) std::memcpy(c->h_stage, edges, eb);
+    if (edges && !staged) VAMP_CK(c, cudaMemcpyAsync(base + c->ar.edges64, edges, eb, cudaMemcpyHostToDevice, c->stream));
+    if (alpha) std::memcpy(c->h_stage + (c->ar.alpha - lo), alpha, kb);
+    if (shift) std::memcpy(c->h_stage + (c->ar.shift - lo), shift, kb);
+    // the pieces that are given, neighbouring ones in one copy
+    const struct { bool on; size_t at, end; } part[3] = {{edges && staged, c->ar.edges64, c->ar.edges64 + eb},
+                                                         {alpha != nullptr, c->ar.alpha, c->ar.alpha + kb},
+                                                         {shift != nullptr, c->ar.shift, c->ar.shift + kb}};
+    for (int i = 0; i < 3;) {
+        if (!part[i].on) { ++i; continue; }
+        int j = i;
+        while (j + 1 < 3 && part[j + 1].on) ++j;
+        VAMP_CK(c, cudaMemcpyAsync(base + part[i].at, c->h_stage + (part[i].at - lo), part[j].end - part[i].at,
+                                   cudaMemcpyHostToDevice, c->stream));
+        i = j + 1;
+    }
+    VAMP_CK(c, vamp::launch_derive(c->prm, c->stream, w_max, n_hist));
+    if (c->uni_on) VAMP_CK(c, vamp::launch_union_build(c->prm, c->stream));
+    VAMP_CK(c, cudaStreamSynchronize(c->stream));
+    c->have_pass = 1;
+    return VAMP_OK;
+}
+
+// Checks of a state that a caller hands in (null: not given).
+vamp_status check_state(vamp_ctx* c, const double* edges, const double* alpha, double w_max)
+{
     const size_t rows = (size_t)c->K * c->d;
     const int n = c->n;
     if (edges) {
@@ -638,16 +688,16 @@ vamp_status vamp_set_state(vamp_ctx* c, const double* edges, const double* alpha
         if (!(s > 0.0)) return fail(c, VAMP_ERR_INVALID_ARG, "alpha must not sum to 0");
     }
     if (!(w_max >= 0.0) || !std::isfinite(w_max)) return fail(c, VAMP_ERR_INVALID_ARG, "w_max must be finite and >= 0");
-    DeviceGuard g(c->dev);
-    if (edges) VAMP_CK(c, cudaMemcpyAsync(c->prm.edges64, edges, rows * (n + 1) * 8, cudaMemcpyHostToDevice, c->stream));
-    if (alpha) VAMP_CK(c, cudaMemcpyAsync(c->prm.alpha, alpha, c->K * 8, cudaMemcpyHostToDevice, c->stream));
-    if (shift) VAMP_CK(c, cudaMemcpyAsync(c->prm.shift, shift, c->K * 8, cudaMemcpyHostToDevice, c->stream));
-    VAMP_CK(c, cudaMemcpyAsync(&c->prm.sc->wmax_gen, &w_max, 8, cudaMemcpyHostToDevice, c->stream));
-    VAMP_CK(c, vamp::launch_derive(c->prm, c->stream));
-    if (c->uni_on) VAMP_CK(c, vamp::launch_union_build(c->prm, c->stream));
-    VAMP_CK(c, cudaStreamSynchronize(c->stream));
-    c->have_pass = 1;
     return VAMP_OK;
+}
+
+}  // namespace
+
+vamp_status vamp_set_state(vamp_ctx* c, const double* edges, const double* alpha, const double* shift, double w_max)
+{
+    if (!c) return VAMP_ERR_INVALID_ARG;
+    const vamp_status s = check_state(c, edges, alpha, w_max);
+    return s != VAMP_OK ? s : upload_state(c, edges, alpha, shift, w_max, -1);
 }
 
 // ---- checkpoint / restore ----------------------------------------------------
@@ -732,22 +782,18 @@ vamp_status vamp_restore(vamp_ctx* c, const void* host_buf, int64_t bytes)
     o += (size_t)c->K * 8;
     std::memcpy(shift.data(), o, (size_t)c->K * 8);
     o += (size_t)c->K * 8;
-    // grids, α, shifts and w_max through the validating state upload
-    vamp_status s = vamp_set_state(c, edges.data(), alpha.data(), shift.data(), h.w_max);
+    const vamp_status s = check_state(c, edges.data(), alpha.data(), h.w_max);
     if (s != VAMP_OK) return s;
-    DeviceGuard g(c->dev);
-    const Params& P = c->prm;
     if (h.n_hist > 0) {
+        DeviceGuard g(c->dev);
+        const Params& P = c->prm;
         VAMP_CK(c, cudaMemcpyAsync(P.sc->hist_I, o, (size_t)h.n_hist * 8, cudaMemcpyHostToDevice, c->stream));
         o += (size_t)h.n_hist * 8;
         VAMP_CK(c, cudaMemcpyAsync(P.sc->hist_V, o, (size_t)h.n_hist * 8, cudaMemcpyHostToDevice, c->stream));
         o += (size_t)h.n_hist * 8;
         VAMP_CK(c, cudaMemcpyAsync(P.sc->hist_comb, o, (size_t)h.n_hist * 4, cudaMemcpyHostToDevice, c->stream));
     }
-    const int32_t nh = h.n_hist;
-    VAMP_CK(c, cudaMemcpyAsync(&P.sc->n_hist, &nh, sizeof nh, cudaMemcpyHostToDevice, c->stream));
-    VAMP_CK(c, cudaStreamSynchronize(c->stream));
-    return VAMP_OK;
+    return upload_state(c, edges.data(), alpha.data(), shift.data(), h.w_max, h.n_hist);
 }
 
 vamp_status vamp_get_pass(vamp_ctx* c, double* D, double* Ic, double* Vc, int64_t* Nc)

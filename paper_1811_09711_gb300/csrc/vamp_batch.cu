@@ -11,6 +11,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -44,6 +45,10 @@ struct vamp_batch {
     int64_t* h_ncalls = nullptr;
     uint32_t* h_iter = nullptr;
     double* h_results = nullptr;
+    std::vector<vamp::Arena> ars;
+    std::vector<size_t> offs;       // of the instances' arenas
+    unsigned char* h_stage = nullptr;  // pinned: one instance's state and scalars
+    std::mutex stage_mu;               // its users (vamp_batch_get_state from several threads)
     // launch shape
     int64_t item_calls = 0;
     int budget_kb = 112;
@@ -79,6 +84,8 @@ vamp_status bfail(vamp_batch* b, vamp_status s, const std::string& msg)
     } while (0)
 
 size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
+
+constexpr size_t STATE_HEAD = offsetof(Scalars, wmax_gen) + sizeof(double);  // of the scalars, for a state's w_max
 
 // Calls per thread of the multi-instance kernel's small-d classes: work
 // items are sized in multiples of PASS_THREADS times this.
@@ -253,6 +260,7 @@ void vamp_batch_destroy(vamp_batch* b)
     cudaFreeHost(b->h_ncalls);
     cudaFreeHost(b->h_iter);
     cudaFreeHost(b->h_results);
+    cudaFreeHost(b->h_stage);
     if (b->stream) cudaStreamDestroy(b->stream);
     if (prev >= 0 && prev != b->dev) cudaSetDevice(prev);
     delete b;
@@ -268,7 +276,8 @@ vamp_status vamp_batch_create(const vamp_config* cfgs, int32_t n, int32_t autotu
     b->n = n;
     b->tune = autotune_tiles ? 1 : 0;
     std::vector<vamp::Setup> setups(n);
-    std::vector<vamp::Arena> ars(n);
+    std::vector<vamp::Arena>& ars = b->ars;
+    ars.resize(n);
     b->prm.resize(n);
     b->cellbuf.assign(n, nullptr);
     b->cellcap.assign(n, 0);
@@ -281,7 +290,9 @@ vamp_status vamp_batch_create(const vamp_config* cfgs, int32_t n, int32_t autotu
     b->pair_off.assign(n + 1, 0);
     b->row_off.assign(n + 1, 0);
     size_t total = 0;
-    std::vector<size_t> offs(n);
+    std::vector<size_t>& offs = b->offs;
+    offs.resize(n);
+    size_t stage = 0;
     for (int i = 0; i < n; ++i) {
         std::string why;
         Params p{};
@@ -296,6 +307,7 @@ vamp_status vamp_batch_create(const vamp_config* cfgs, int32_t n, int32_t autotu
         ars[i] = vamp::plan_arena(p);
         offs[i] = total;
         total += a256(ars[i].bytes);
+        stage = std::max(stage, ars[i].sc + STATE_HEAD);
         b->combine_from[i] = cfgs[i].combine_from;
         b->K[i] = p.K;
         b->d[i] = p.d;
@@ -339,6 +351,7 @@ vamp_status vamp_batch_create(const vamp_config* cfgs, int32_t n, int32_t autotu
     if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_ncalls, (size_t)n * 8);
     if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_iter, (size_t)n * 4);
     if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_results, (size_t)n * 9 * 8);
+    if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_stage, stage);
     if (e != cudaSuccess) {
         vamp_batch_destroy(b);
         return e == cudaErrorMemoryAllocation ? VAMP_ERR_OOM : VAMP_ERR_CUDA;
@@ -370,7 +383,7 @@ vamp_status vamp_batch_create(const vamp_config* cfgs, int32_t n, int32_t autotu
             for (int j = 0; j <= P.n; ++j) edges[r * (P.n + 1) + j] = (double)j / (double)P.n;
         BCREATE(cudaMemcpyAsync(P.edges64, edges.data(), edges.size() * 8, cudaMemcpyHostToDevice, b->stream));
         BCREATE(cudaMemcpyAsync(P.alpha, alpha.data(), P.K * 8, cudaMemcpyHostToDevice, b->stream));
-        BCREATE(vamp::upload_setup(P, setups[i], b->stream));
+        BCREATE(vamp::upload_setup(P, setups[i], b->stream, false));
         BCREATE(vamp::launch_derive(P, b->stream));
         BCREATE(cudaStreamSynchronize(b->stream));  // host vectors go out of scope
     }
@@ -471,13 +484,18 @@ vamp_status vamp_batch_get_state(vamp_batch* b, int32_t instance, double* edges,
                                  double* w_max)
 {
     if (!b || instance < 0 || instance >= b->n) return VAMP_ERR_INVALID_ARG;
+    // the state is one range of the instance's arena: one copy to pinned memory
     const Params& P = b->prm[instance];
-    const size_t rows = (size_t)P.K * P.d;
-    if (edges) BCK(b, cudaMemcpyAsync(edges, P.edges64, rows * (P.n + 1) * 8, cudaMemcpyDeviceToHost, b->stream));
-    if (alpha) BCK(b, cudaMemcpyAsync(alpha, P.alpha, P.K * 8, cudaMemcpyDeviceToHost, b->stream));
-    if (shift) BCK(b, cudaMemcpyAsync(shift, P.shift, P.K * 8, cudaMemcpyDeviceToHost, b->stream));
-    if (w_max) BCK(b, cudaMemcpyAsync(w_max, &P.sc->wmax_gen, 8, cudaMemcpyDeviceToHost, b->stream));
+    const vamp::Arena& A = b->ars[instance];
+    const size_t eb = (size_t)P.K * P.d * (P.n + 1) * 8, kb = (size_t)P.K * 8, lo = edges ? A.edges64 : A.alpha;
+    std::lock_guard<std::mutex> lk(b->stage_mu);
+    BCK(b, cudaMemcpyAsync(b->h_stage, (unsigned char*)b->arena + b->offs[instance] + lo, A.sc + STATE_HEAD - lo,
+                           cudaMemcpyDeviceToHost, b->stream));
     BCK(b, cudaStreamSynchronize(b->stream));
+    if (edges) std::memcpy(edges, b->h_stage, eb);
+    if (alpha) std::memcpy(alpha, b->h_stage + (A.alpha - lo), kb);
+    if (shift) std::memcpy(shift, b->h_stage + (A.shift - lo), kb);
+    if (w_max) *w_max = reinterpret_cast<const Scalars*>(b->h_stage + (A.sc - lo))->wmax_gen;
     return VAMP_OK;
 }
 

@@ -249,12 +249,6 @@ template <> struct Prec<double> {
     static __device__ __forceinline__ double gk2(const Params& P) { return P.gk2; }
     // in-bin fraction of the forward map: the exact 33-bit value
     static __device__ __forceinline__ double frac(uint64_t low33) { return sf_frac33(low33); }
-    // in-bin fraction of a stratified call: remainder over n_r 2^33, one
-    // correctly rounded division
-    static __device__ __forceinline__ double frac_div(uint64_t rem, uint64_t den)
-    {
-        return __ddiv_rn((double)rem, (double)den);
-    }
     // x = ξ_j + frac (ξ_{j+1} - ξ_j), rounded as two separate operations
     static __device__ __forceinline__ double lerp(double e0, double e1, double fr)
     {
@@ -332,10 +326,6 @@ template <> struct Prec<float> {
     static __device__ __forceinline__ float gk2(const Params& P) { return P.gk2_f; }
     // top 24 bits of the 33-bit fraction (exact conversion)
     static __device__ __forceinline__ float frac(uint64_t low33) { return (float)(uint32_t)(low33 >> 9) * 0x1p-24f; }
-    static __device__ __forceinline__ float frac_div(uint64_t rem, uint64_t den)
-    {
-        return (float)__ddiv_rn((double)rem, (double)den);
-    }
     static __device__ __forceinline__ float lerp(float e0, float e1, float fr) { return fmaf(fr, e1 - e0, e0); }
     static __device__ __forceinline__ float tan_(float v) { return tanf(v); }
     static __device__ __forceinline__ float atan_(float v) { return atanf(v); }
@@ -464,6 +454,22 @@ __device__ __forceinline__ int lookup(const SH& sh, const unsigned char* row, in
     return j;
 }
 
+// Forward bin j and in-bin fraction of a stratified call from the integer t
+// below n n_r 2^33: t = (j n_r + rest) 2^33 + low, fraction (rest 2^33 + low) /
+// (n_r 2^33) to about 2^-53 by the integer reciprocal of n_r.  (64-bit integer
+// and FP64 divisions here were a third of a d = 4 stratified pass.)
+template <typename T>
+__device__ __forceinline__ T strat_fraction(uint64_t t, uint32_t nr, Sf inv_nr, int& j)
+{
+    const uint32_t hi = (uint32_t)(t >> 33), q = hi / nr;  // below n n_r < 2^28
+    j = (int)q;
+    if (nr == 1u) return Prec<T>::frac(t & ((1ull << 33) - 1ull));
+    const uint64_t rem = ((uint64_t)(hi - q * nr) << 33) | (t & ((1ull << 33) - 1ull));
+    if (rem == 0ull) return T(0);
+    const int z = __clzll((long long)rem);
+    return (T)sf_to_double(sf_norm(sf_mul(Sf{rem << z, -z}, Sf{inv_nr.m, inv_nr.e - 33})));
+}
+
 // ---------------------------------------------------------------------------
 // Forward map of the selected channel (lookup block in global memory):
 // r -> x_c -> p, the own term g_c(x_c)/φ'_c(x_c) and the Gaussian exponent
@@ -476,6 +482,7 @@ __device__ __forceinline__ void forward_call(const Params& P, const SH& sh, int 
 {
     const int d = sh.d(), n = sh.n();
     const unsigned char* blk = Prec<T>::lk(P) + (size_t)c * sh.bytes();
+    const Sf inv_nr = dig ? sf_rcp(sf_from_double((double)nr)) : Sf{0, 0};
     T g = T(1);
 #pragma unroll
     for (int k = 0; k < SH::DM; ++k) {
@@ -485,11 +492,8 @@ __device__ __forceinline__ void forward_call(const Params& P, const SH& sh, int 
             if (dig) {
                 // stratified call: r_k = (a_k + u_k) / n_r, from the integer
                 // (2^33 a_k + 2X + 1) n over n_r 2^33 (n_r = 1: the line below)
-                const uint64_t den = (uint64_t)nr << 33;
                 const uint64_t t = (((uint64_t)dig[k] << 33) + 2ull * X[k] + 1ull) * (uint64_t)n;
-                const uint64_t jj = t / den;
-                j = (int)jj;
-                fr = Prec<T>::frac_div(t - jj * den, den);
+                fr = strat_fraction<T>(t, nr, inv_nr, j);
             } else {
                 const uint64_t t = (2ull * X[k] + 1ull) * (uint64_t)n;
                 j = (int)(t >> 33);
@@ -701,6 +705,7 @@ __device__ __forceinline__ void soft_forward(const Params& P, const SH& sh, int 
     const unsigned char* blk = P.lk64 + (size_t)c * sh.bytes();
     const ChanHdr<double>* h = reinterpret_cast<const ChanHdr<double>*>(blk);
     const double* e0 = P.edges64 + (size_t)c * d * (size_t)(n + 1);
+    const Sf inv_nr = digit ? sf_rcp(sf_from_double((double)nr)) : Sf{0, 0};
     uint64_t acc = 1ull << 63;
     int ae = 0;  // acc 2^(ae - 1022 d - 63)
 #pragma unroll
@@ -711,11 +716,8 @@ __device__ __forceinline__ void soft_forward(const Params& P, const SH& sh, int 
             if (digit) {
                 // stratified call: r_k = (a_k + u_k) / n_r, from the integer
                 // (2^33 a_k + 2X + 1) n over n_r 2^33 (n_r = 1: the line below)
-                const uint64_t den = (uint64_t)nr << 33;
                 const uint64_t t = (((uint64_t)digit[k] << 33) + 2ull * X[k] + 1ull) * (uint64_t)n;
-                const uint64_t jj = t / den;
-                jf[k] = (int)jj;
-                fr = Prec<double>::frac_div(t - jj * den, den);
+                fr = strat_fraction<double>(t, nr, inv_nr, jf[k]);
             } else {
                 const uint64_t t = (2ull * X[k] + 1ull) * (uint64_t)n;
                 jf[k] = (int)(t >> 33);

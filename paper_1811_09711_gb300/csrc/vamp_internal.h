@@ -103,8 +103,10 @@ struct Arena {
 };
 Arena plan_arena(const Params& P);
 void bind_arena(Params& P, unsigned char* base, const Arena& A);  // sets every array pointer
-// Copies headers and peak records into the arena (async on s).
-cudaError_t upload_setup(const Params& P, const Setup& S, cudaStream_t s);
+// Copies headers and peak records into the arena (async on s): those of the
+// evaluation precision, and the other precision's headers where `both` (the
+// interval tables take their maps from the FP64 ones).
+cudaError_t upload_setup(const Params& P, const Setup& S, cudaStream_t s, bool both);
 
 // Shared-memory layout of a staged-tile pass kernel: channels per tile, log2
 // of the copies of the d-values, bytes of the integration and generation form.
@@ -172,7 +174,9 @@ const void* pass_multi_kernel(int fp32, int minb, int strat = 0);
 cudaError_t launch_begin_pass(const Params& P, int64_t N, cudaStream_t s, int clear = 0, int64_t cells = 0);
 cudaError_t launch_finish_pass(const Params& P, int combine, cudaStream_t s);
 cudaError_t launch_strat_q(const Params& P, cudaStream_t s);  // stratified passes, before finish
-cudaError_t launch_derive(const Params& P, cudaStream_t s);
+// w_max >= 0 also sets the generation maximum, n_hist >= 0 the length of the
+// history of passes.
+cudaError_t launch_derive(const Params& P, cudaStream_t s, double w_max = -1.0, int n_hist = -1);
 cudaError_t launch_refine(const Params& P, cudaStream_t s);
 cudaError_t launch_update_alpha(const Params& P, cudaStream_t s);
 cudaError_t launch_pass_result(const Params& P, double* out, cudaStream_t s);  // 9 doubles

@@ -82,6 +82,22 @@ __device__ __forceinline__ double block_sum(double v, double* tmp)
     return s;
 }
 
+// Two sums at once.
+__device__ __forceinline__ void block_sum2(double& u, double& v, double (*tmp)[2])
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        u += __shfl_xor_sync(0xffffffffu, u, o);
+        v += __shfl_xor_sync(0xffffffffu, v, o);
+    }
+    __syncthreads();
+    if (lane == 0) { tmp[wid][0] = u; tmp[wid][1] = v; }
+    __syncthreads();
+    u = v = 0.0;
+    for (int q = 0; q < nw; ++q) { u += tmp[q][0]; v += tmp[q][1]; }
+}
+
 __device__ __forceinline__ double lanes_sum(double v)
 {
 #pragma unroll
@@ -184,9 +200,21 @@ __global__ void k_begin_pass(Params P, int64_t N, int clear, int64_t cells)
 // all, the combination of the passes by the first warp.
 __device__ void finish_pass_dev(const Params& P, int combine)
 {
-    __shared__ double tmp[33];
+    __shared__ double tmp[32][2];
     Scalars* sc = P.sc;
     double I = 0.0, V = 0.0;
+    // this lane's share of the history of passes, fetched while the channels' sums are on their way
+    const int h = sc->n_hist;
+    const unsigned long long wbits = sc->wmax_bits;
+    double cnt = 0.0, nzero = 0.0, zI = 0.0, sw = 0.0, swi = 0.0;
+    auto take = [&](double hI, double hV) {
+        cnt += 1.0;
+        if (hV <= 0.0) { nzero += 1.0; zI += hI; }
+        else { const double iv = 1.0 / hV; sw += iv; swi += hI * iv; }
+    };
+    if (threadIdx.x < 32)
+        for (int q = threadIdx.x; q < h; q += 32)
+            if (sc->hist_comb[q]) take(sc->hist_I[q], sc->hist_V[q]);
     for (int c = threadIdx.x; c < P.K; c += blockDim.x) {
         const int64_t nci = P.Nc[c];
         if (nci == 0) { P.Ic[c] = P.Vc[c] = P.Wc[c] = 0.0; P.shift[c] = 0.0; continue; }
@@ -209,28 +237,17 @@ __device__ void finish_pass_dev(const Params& P, int combine)
         I += al * Ic;
         V += al * al * Vv / Nc;
     }
-    I = block_sum(I, tmp);
-    V = block_sum(V, tmp);
+    block_sum2(I, V, tmp);
     if (threadIdx.x >= 32) return;
     const int lane = threadIdx.x;
-    // the passes so far and this one
-    const int h = sc->n_hist, nh = h < 1024 ? h + 1 : h;
     if (lane == 0 && h < 1024) {
         sc->hist_I[h] = I;
         sc->hist_V[h] = V;
         sc->hist_comb[h] = combine;
         sc->n_hist = h + 1;
+        if (combine) take(I, V);
     }
-    __syncwarp();
     // inverse-variance combination of the flagged passes
-    double cnt = 0.0, nzero = 0.0, zI = 0.0, sw = 0.0, swi = 0.0;
-    for (int q = lane; q < nh; q += 32) {
-        if (!sc->hist_comb[q]) continue;
-        const double hI = sc->hist_I[q], hV = sc->hist_V[q];
-        cnt += 1.0;
-        if (hV <= 0.0) { nzero += 1.0; zI += hI; }
-        else { const double iv = 1.0 / hV; sw += iv; swi += hI / hV; }
-    }
     cnt = lanes_sum(cnt);
     double cI = 0.0, cS = 0.0, chi = 0.0;
     if (cnt > 0.0) {
@@ -243,17 +260,18 @@ __device__ void finish_pass_dev(const Params& P, int combine)
             cS = sqrt(1.0 / sw);
             if (cnt > 1.0) {
                 double ch = 0.0;
-                for (int q = lane; q < nh; q += 32) {
+                for (int q = lane; q < h; q += 32) {
                     if (!sc->hist_comb[q]) continue;
                     const double dI = sc->hist_I[q] - cI;
                     ch += dI * dI / sc->hist_V[q];
                 }
+                if (lane == 0 && h < 1024 && combine) ch += (I - cI) * (I - cI) / V;
                 chi = lanes_sum(ch) / (cnt - 1.0);
             }
         }
     }
     if (lane != 0) return;
-    const double wmax = __longlong_as_double((long long)sc->wmax_bits);
+    const double wmax = __longlong_as_double((long long)wbits);
     sc->wmax_gen = wmax;
     sc->res[0] = I;
     sc->res[1] = V;
@@ -378,7 +396,7 @@ __device__ __forceinline__ void store_alpha(const Params& P, int c, double a)
     P.alphaN[c] = a * reinterpret_cast<const ChanHdr<double>*>(P.lk64 + (size_t)c * P.lay64.bytes)->gN;
 }
 
-__global__ void k_derive(Params P)
+__global__ void k_derive(Params P, double w_max, int n_hist)
 {
     extern __shared__ int dq0[];
     const int rows = P.K * P.d;
@@ -387,8 +405,11 @@ __global__ void k_derive(Params P)
     const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int nw = gridDim.x * (blockDim.x >> 5);
     for (int row = w; row < rows; row += nw) derive_row(P, row, lane, P.edges64 + (size_t)row * (P.n + 1), q0);
-    if (blockIdx.x == 0)
+    if (blockIdx.x == 0) {
         for (int c = threadIdx.x; c < P.K; c += blockDim.x) store_alpha(P, c, P.alpha[c]);
+        if (threadIdx.x == 0 && w_max >= 0.0) P.sc->wmax_gen = w_max;
+        if (threadIdx.x == 0 && n_hist >= 0) P.sc->n_hist = n_hist;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -526,7 +547,7 @@ __global__ void __launch_bounds__(REFINE_WARPS * 32) k_refine(Params P)
 // terms α_c ω_c^β and then the new weights between the sums).
 __device__ void update_alpha_dev(const Params& P)
 {
-    __shared__ double tmp[33];
+    __shared__ double tmp[33], tmp2[32][2];
     const int K = P.K;
     auto omega = [&](int c) { return P.omega_mode ? P.Wc[c] : P.Vc[c]; };
     double SU = 0.0, MU = 0.0;
@@ -541,8 +562,7 @@ __device__ void update_alpha_dev(const Params& P)
         }
         P.Acum[c] = u;
     }
-    SU = block_sum(SU, tmp);
-    MU = block_sum(MU, tmp);
+    block_sum2(SU, MU, tmp2);
     double tot = 0.0;
     for (int c = threadIdx.x; c < K; c += blockDim.x) {
         double a = P.alpha[c];
@@ -884,6 +904,9 @@ cudaError_t launch_wait_selftest(long long limit, unsigned int* flag, long long*
 // ---------------------------------------------------------------------------
 // host-side launchers
 // ---------------------------------------------------------------------------
+// Threads of the one-block kernels: a channel a thread up to 256.
+static int small_block(int K) { return std::min(256, (K + 31) / 32 * 32); }
+
 cudaError_t launch_begin_pass(const Params& P, int64_t N, cudaStream_t s, int clear, int64_t cells)
 {
     // a block for every 4096 words to clear, up to two per SM
@@ -901,15 +924,15 @@ cudaError_t launch_strat_q(const Params& P, cudaStream_t s)
 
 cudaError_t launch_finish_pass(const Params& P, int combine, cudaStream_t s)
 {
-    k_finish_pass<<<1, 256, 0, s>>>(P, combine);
+    k_finish_pass<<<1, small_block(P.K), 0, s>>>(P, combine);
     return cudaGetLastError();
 }
 
-cudaError_t launch_derive(const Params& P, cudaStream_t s)
+cudaError_t launch_derive(const Params& P, cudaStream_t s, double w_max, int n_hist)
 {
     const int rows = P.K * P.d;
     const int blocks = min((rows + 3) / 4, 1024);
-    k_derive<<<blocks, 128, (size_t)4 * (P.n + 1) * sizeof(int), s>>>(P);
+    k_derive<<<blocks, 128, (size_t)4 * (P.n + 1) * sizeof(int), s>>>(P, w_max, n_hist);
     return cudaGetLastError();
 }
 
@@ -930,13 +953,13 @@ cudaError_t launch_pass_result(const Params& P, double* out, cudaStream_t s)
 
 cudaError_t launch_update_alpha(const Params& P, cudaStream_t s)
 {
-    k_update_alpha<<<1, 256, 0, s>>>(P);
+    k_update_alpha<<<1, small_block(P.K), 0, s>>>(P);
     return cudaGetLastError();
 }
 
 cudaError_t launch_gen_prepare(const Params& P, cudaStream_t s)
 {
-    k_gen_prepare<<<1, P.K > 128 ? 256 : (P.K + 31) / 32 * 32, 0, s>>>(P);
+    k_gen_prepare<<<1, small_block(P.K), 0, s>>>(P);
     return cudaGetLastError();
 }
 

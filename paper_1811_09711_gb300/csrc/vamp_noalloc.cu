@@ -135,7 +135,7 @@ extern "C" vamp_status vamp_sample_pass_static(const vamp_config* cfg, const dou
     // what must start from zero: the scalars (the pass accumulators: launch_begin_pass)
     e = cudaMemsetAsync(pr.sc, 0, sizeof(Scalars), stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(pr.shift, dev_shift, K * 8, cudaMemcpyDeviceToDevice, stream);
-    if (e == cudaSuccess) e = vamp::upload_setup(pr, S, stream);
+    if (e == cudaSuccess) e = vamp::upload_setup(pr, S, stream, false);
     if (e == cudaSuccess) e = vamp::launch_derive(pr, stream);
     if (e == cudaSuccess) e = vamp::launch_begin_pass(pr, n_calls, stream, 1);
     if (e == cudaSuccess) {

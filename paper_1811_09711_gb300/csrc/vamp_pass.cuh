@@ -141,11 +141,15 @@ __device__ __forceinline__ void phase_a(const Params& P, const SH& sh, uint32_t 
         if (strat) {
             // cell of the call and its base-n_r digits (§3.3)
             nr = (uint32_t)P.nr[c];
-            uint32_t cell = (uint32_t)(((C.valid[q] ? i : base) - P.Pc[c]) / P.spc[c]);
+            uint32_t cell = (uint32_t)((C.valid[q] ? i : base) - P.Pc[c]) / (uint32_t)P.spc[c];  // both < 2^32
 #pragma unroll
             for (int k = 0; k < DM; ++k) {
-                dig[k] = cell % nr;
-                cell /= nr;
+                dig[k] = 0u;
+                if (sh.has(k)) {
+                    const uint32_t up = cell / nr;
+                    dig[k] = cell - up * nr;
+                    cell = up;
+                }
             }
         }
         if constexpr (sizeof(T) == 8) {
@@ -237,7 +241,7 @@ __device__ __forceinline__ void phase_c_int(const SH& sh, const Calls<T, CPT, SH
         s1 += dv;
         s2 += dv * dv;
         if (cs.sum)  // stratified: the sum of the call's cell
-            atomicAdd(&cs.sum[cs.coff + (cs.l0 + call_of<CPT>(q)) / cs.spc], dv);
+            atomicAdd(&cs.sum[cs.coff + (uint32_t)(cs.l0 + call_of<CPT>(q)) / (uint32_t)cs.spc], dv);
         wm = max_abs(wm, w);  // signed integrands: w_max bounds |w|
         const double w2 = w * w;
 #pragma unroll

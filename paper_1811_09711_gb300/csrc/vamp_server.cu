@@ -232,7 +232,7 @@ vamp_status admit(vamp_server* s, Req* r)
     if (e == cudaSuccess) e = cudaMemsetAsync(r->mem, 0, r->ar.bytes, r->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(P.edges64, edges.data(), edges.size() * 8, cudaMemcpyHostToDevice, r->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(P.alpha, alpha.data(), P.K * 8, cudaMemcpyHostToDevice, r->stream);
-    if (e == cudaSuccess) e = vamp::upload_setup(P, r->S, r->stream);
+    if (e == cudaSuccess) e = vamp::upload_setup(P, r->S, r->stream, false);
     if (e == cudaSuccess) e = vamp::launch_derive(P, r->stream);
     if (e == cudaSuccess) e = cudaEventRecord(r->ev, r->stream);  // setup done (polled)
     if (e != cudaSuccess) return VAMP_ERR_CUDA;

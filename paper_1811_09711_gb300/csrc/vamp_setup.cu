@@ -277,13 +277,15 @@ Arena plan_arena(const Params& P)
     const size_t K = (size_t)P.K, rows = K * P.d;
     size_t off = 0;
     auto take = [&](size_t bytes) { const size_t o = off; off += a256(bytes); return o; };
+    // the state that callers read and write, and the scalars: one range
     A.edges64 = take(rows * (P.n + 1) * 8);
+    A.alpha = take(K * 8);
+    A.shift = take(K * 8);
+    A.sc = take(sizeof(Scalars));
     A.lk64 = take(K * P.lay64.bytes);
     A.lk32 = take(K * P.lay32.bytes);
-    A.alpha = take(K * 8);
     A.alpha32 = take(K * 4);
     A.alphan = take(K * 8);
-    A.shift = take(K * 8);
     A.acum = take(K * 8);
     A.nc = take(K * 8);
     A.pc = take((K + 1) * 8);
@@ -294,7 +296,6 @@ Arena plan_arena(const Params& P)
     A.wc = take(K * 8);
     A.pk64 = take((size_t)P.P * sizeof(MapRec<double>));
     A.pk32 = take((size_t)P.P * sizeof(MapRec<float>));
-    A.sc = take(sizeof(Scalars));
     A.nr = take(K * 8);
     A.spc = take(K * 8);
     A.coff = take((K + 1) * 8);
@@ -334,16 +335,19 @@ void bind_arena(Params& P, unsigned char* b, const Arena& A)
     P.eq_ent = P.n_eq_ent > 0 ? (const int32_t*)(b + A.eqent) : nullptr;
 }
 
-cudaError_t upload_setup(const Params& P, const Setup& S, cudaStream_t s)
+cudaError_t upload_setup(const Params& P, const Setup& S, cudaStream_t s, bool both)
 {
-    cudaError_t e = cudaMemcpy2DAsync(P.lk64, P.lay64.bytes, S.hdr64.data(), P.lay64.H, P.lay64.H, P.K,
-                                      cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess)
+    cudaError_t e = cudaSuccess;
+    if (both || !P.fp32)
+        e = cudaMemcpy2DAsync(P.lk64, P.lay64.bytes, S.hdr64.data(), P.lay64.H, P.lay64.H, P.K,
+                              cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess && (both || P.fp32))
         e = cudaMemcpy2DAsync(P.lk32, P.lay32.bytes, S.hdr32.data(), P.lay32.H, P.lay32.H, P.K,
                               cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess)
+    // peaks of their own (matching ones are in the channels' headers)
+    if (e == cudaSuccess && !P.matching && !P.fp32)
         e = cudaMemcpyAsync((void*)P.pk64, S.pk64.data(), S.pk64.size(), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess)
+    if (e == cudaSuccess && !P.matching && P.fp32)
         e = cudaMemcpyAsync((void*)P.pk32, S.pk32.data(), S.pk32.size(), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess && P.n_eq_ent > 0)
         e = cudaMemcpyAsync((void*)P.eq_off, S.eq_off.data(), S.eq_off.size() * 4, cudaMemcpyHostToDevice, s);

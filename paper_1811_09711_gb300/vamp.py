@@ -205,17 +205,24 @@ def _ptr(a):
     return None if a is None else a.ctypes.data_as(C.c_void_p)
 
 
+# MapDesc as a numpy record (its layout is checked below)
+_MAP_DTYPE = np.dtype([("n_mapped", np.int32), ("coord", np.int32, 4), ("kind", np.int32, 4),
+                       ("a", np.float64, 4), ("b", np.float64, 4)], align=True)
+assert _MAP_DTYPE.itemsize == C.sizeof(MapDesc) and all(
+    _MAP_DTYPE.fields[f][1] == getattr(MapDesc, f).offset for f, _ in MapDesc._fields_)
+
+
 def _map_array(ms) -> C.Array:
-    arr = (MapDesc * len(ms))()
-    for q in range(len(ms)):
-        r = arr[q]
-        r.n_mapped = int(ms.n_mapped[q])
-        for s in range(4):
-            r.coord[s] = int(ms.coord[q, s])
-            r.kind[s] = int(ms.kind[q, s])
-            r.a[s] = float(ms.a[q, s])
-            r.b[s] = float(ms.b[q, s])
-    return arr
+    """The maps as an array of MapDesc, filled a field at a time (a slot at a
+    time took 45 us for six channels and six peaks)."""
+    k = len(ms)
+    if k == 0:
+        return (MapDesc * 0)()
+    rec = np.zeros(k, _MAP_DTYPE)
+    rec["n_mapped"] = ms.n_mapped
+    for f in ("coord", "kind", "a", "b"):
+        rec[f] = getattr(ms, f)[:, :4]
+    return (MapDesc * k).from_buffer(rec)
 
 
 def make_config(problem, precision: int = PREC_FP64):
