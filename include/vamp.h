@@ -308,15 +308,17 @@ typedef struct vamp_pipe_peaks {
 vamp_status vamp_measure_peaks(vamp_pipe_peaks *out);
 
 /* Name of the pass kernel the context uses for mode 0 (integration) or 1
- * (generation), as profilers print it, e.g. "k_pass<float, 0, 2, 14, 100, 2>",
+ * (generation), as profilers print it, e.g. "k_pass<float, 0, 2, 14, 100, 2>"
+ * (a kernel for a range of d, printed by profilers as k_pass_dims or
+ * k_union_dims, has the range in the place of d: "k_pass<float, 0, 2, 5-8, 0, 2>"),
  * written NUL-terminated into buf (len bytes, host).  INVALID_ARG for a bad
  * mode or a buffer too small. */
 vamp_status vamp_pass_kernel_name(const vamp_ctx *ctx, int32_t mode, char *buf, int32_t len);
 
 /* Number of compiled pass-kernel variants that can run this context's shape
  * and sampling mode: the autotuner's candidates, in a fixed order
- * (shape-specialised staged-tile kernels "k_pass" first, then the generic
- * one; for FP32-eval importance sampling with K <= 64 and K (n+1) <= 16384,
+ * (staged-tile kernels "k_pass" for the exact shape first, then for the range
+ * of d, then for any shape; for FP32-eval importance sampling with K <= 64 and K (n+1) <= 16384,
  * then the union kernels "k_union", which find every channel's bin of p_k
  * with one search in per-coordinate tables of all channels' edge images,
  * Eq. 30 evaluated the same way). */

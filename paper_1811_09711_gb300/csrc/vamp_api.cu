@@ -244,9 +244,10 @@ vamp_status choose_variant(vamp_ctx* c, int64_t n_calls)
         *grid = (b > 0 ? b : 1) * c->sm_count;
         return e;
     };
-    const int64_t probe = std::min<int64_t>(std::max<int64_t>(n_calls, 1 << 16), 1 << 24);
     int nclass = 0;
-    while ((int64_t(1) << (nclass + 1)) <= probe) ++nclass;
+    while ((int64_t(1) << (nclass + 1)) <= std::min<int64_t>(std::max<int64_t>(n_calls, 1 << 16), 1 << 24)) ++nclass;
+    // 2^21 calls rank the kernels as more do, in a fraction of the time
+    const int64_t probe = std::min<int64_t>(std::max<int64_t>(n_calls, 1 << 16), 1 << 21);
     const auto key = std::make_tuple(c->dev, c->fp32, c->d, c->n, std::min(c->K, 64), nclass, c->prm.stratified);
     const PassVariant* best = nullptr;
     {
@@ -258,9 +259,9 @@ vamp_status choose_variant(vamp_ctx* c, int64_t n_calls)
     // FP64: the kernel of the range of d was the faster one at every size measured
     if (!best && (cand.size() == 1 || !c->fp32)) best = cand[0];
     if (!best) {
-        // time each candidate on a pass of `probe` calls over the current
-        // grids; the pass result is discarded (no finish kernel runs) and
-        // the accumulators are cleared again below
+        // time candidates on a pass of `probe` calls over the current grids;
+        // the pass result is discarded (no finish kernel runs) and the
+        // accumulators are cleared again below
         for (const PassVariant* v : cand)
             if (v->uni && !c->uni_on) {
                 const vamp_status us = union_enable(c);
@@ -270,7 +271,7 @@ vamp_status choose_variant(vamp_ctx* c, int64_t n_calls)
         VAMP_CK(c, cudaEventCreate(&e0));
         VAMP_CK(c, cudaEventCreate(&e1));
         float best_ms = 1e30f;
-        for (const PassVariant* v : cand) {
+        auto time_one = [&](const PassVariant* v, float* ms) -> vamp_status {
             int grid = 0;
             VAMP_CK(c, grid_of(v, 0, &grid));
             const vamp::TilePlan s = shape_of(c, v);
@@ -278,17 +279,40 @@ vamp_status choose_variant(vamp_ctx* c, int64_t n_calls)
             A.tile = s.tile;
             A.ntiles = (c->K + s.tile - 1) / s.tile;
             A.dshift = s.dshift;
-            float ms_v = 0.f;
             for (int rep = 0; rep < 2; ++rep) {
                 VAMP_CK(c, vamp::launch_begin_pass(c->prm, probe, c->stream));
                 VAMP_CK(c, cudaEventRecord(e0, c->stream));
                 VAMP_CK(c, v->launch(c->prm, 0, A, grid, s.smem_int, c->stream));
                 VAMP_CK(c, cudaEventRecord(e1, c->stream));
                 VAMP_CK(c, cudaEventSynchronize(e1));
-                VAMP_CK(c, cudaEventElapsedTime(&ms_v, e0, e1));
+                VAMP_CK(c, cudaEventElapsedTime(ms, e0, e1));
             }
-            if (ms_v < best_ms) { best_ms = ms_v; best = v; }
+            return VAMP_OK;
+        };
+        auto contest = [&](auto&& enters) -> vamp_status {
+            for (const PassVariant* v : cand) {
+                if (!enters(v)) continue;
+                float ms = 0.f;
+                const vamp_status ts = time_one(v, &ms);
+                if (ts != VAMP_OK) return ts;
+                if (ms < best_ms) { best_ms = ms; best = v; }
+            }
+            return VAMP_OK;
+        };
+        // The two families round differently at bin edges (the union pass
+        // decides a bin exactly for its FP32 p), so which one a problem gets
+        // is settled between their exact-shape and any-shape kernels; the
+        // kernels of a range of d then compete within that family, and do not
+        // move a problem from the more exact one to the other by being faster.
+        vamp_status ts;
+        if (any_uni && !reduced) {
+            ts = contest([](const PassVariant* v) { return v->dhi == 0; });
+            const int family = best ? best->uni : 0;
+            if (ts == VAMP_OK) ts = contest([&](const PassVariant* v) { return v->dhi > 0 && v->uni == family; });
+        } else {
+            ts = contest([](const PassVariant* v) { return v->D > 0 || v->dhi > 0; });
         }
+        if (ts != VAMP_OK) return ts;
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
         // the probe touched the accumulators and the pass scalars (not the
@@ -909,8 +933,11 @@ vamp_status vamp_pass_kernel_name(const vamp_ctx* c, int32_t mode, char* buf, in
 {
     if (!c || !c->var || (mode != 0 && mode != 1) || !buf || len < 1) return VAMP_ERR_INVALID_ARG;
     const vamp::PassVariant* v = c->var;
-    const int k = std::snprintf(buf, (size_t)len, "%s<%s, %d, %d, %d, %d, %d>", v->family,
-                                v->fp32 ? "float" : "double", mode, v->cpt, v->D, v->NB, v->minb);
+    char dims[24];
+    if (v->dhi > 0) std::snprintf(dims, sizeof dims, "%d-%d", v->dlo, v->dhi);
+    else std::snprintf(dims, sizeof dims, "%d", v->D);
+    const int k = std::snprintf(buf, (size_t)len, "%s<%s, %d, %d, %s, %d, %d>", v->family,
+                                v->fp32 ? "float" : "double", mode, v->cpt, dims, v->NB, v->minb);
     return (k < 0 || k >= len) ? VAMP_ERR_INVALID_ARG : VAMP_OK;
 }
 

@@ -70,6 +70,7 @@ void add_pass_variants_f32_dims(std::vector<PassVariant>& v);
 void add_pass_variants_f64(std::vector<PassVariant>& v);
 void add_pass_variants_f64_dims(std::vector<PassVariant>& v);
 void add_pass_variants_union(std::vector<PassVariant>& v);
+void add_pass_variants_union_dims(std::vector<PassVariant>& v);
 
 // ---- interval tables of the union pass (vamp_union.cu) -----------------------
 // Whether the union kernels take a problem of this kind: FP32-eval,
@@ -122,8 +123,8 @@ TilePlan plan_tiles(size_t S, int K, int dn, size_t fixed, size_t budget);
 // of the current device.
 TilePlan pass_smem(const Params& P, int fp32, int minb = 2);
 // Candidate kernels for a shape: exact (D, NB) matches first, then those of
-// its range of d (pseudo-stratified passes: the any-shape form, which alone
-// carries the cell code);
+// its range of d, then the any-shape form (pseudo-stratified passes: that one
+// alone, which carries the cell code);
 // with the channel count K given (K > 0) and union_fits, the union kernels
 // after them (exact shape first).
 std::vector<const PassVariant*> pass_candidates(int fp32, int d, int n, int stratified = 0, int K = 0);

@@ -402,28 +402,19 @@ std::vector<const PassVariant*> pass_candidates(int fp32, int d, int n, int stra
         add_pass_variants_f64(all);
         add_pass_variants_f64_dims(all);
         add_pass_variants_union(all);
+        add_pass_variants_union_dims(all);
     });
     const bool uni = K > 0 && union_fits(fp32, d, K, n, stratified);
-    std::vector<const PassVariant*> exact, generic, uexact, ugeneric;
-    for (const PassVariant& v : all) {
-        if (v.fp32 != fp32) continue;
-        if (v.uni) {
-            if (!uni) continue;
-            if (v.D == d && v.NB == n) uexact.push_back(&v);
-            else if (v.D == 0 && v.NB == 0) ugeneric.push_back(&v);
-            continue;
-        }
-        if (v.D == d && v.NB == n && !stratified) exact.push_back(&v);
-        else if (v.D == 0 && v.NB == 0 && (stratified ? v.dhi == 0 : v.dlo <= d && d <= v.dhi)) generic.push_back(&v);
-    }
-    // FP64: the any-shape form stays selectable behind the kernel of the range
-    if (!fp32 && !stratified)
-        for (const PassVariant& v : all)
-            if (!v.fp32 && v.D == 0 && v.NB == 0 && v.dhi == 0) generic.push_back(&v);
-    for (const PassVariant* v : generic) exact.push_back(v);
-    for (const PassVariant* v : uexact) exact.push_back(v);
-    for (const PassVariant* v : ugeneric) exact.push_back(v);
-    return exact;
+    std::vector<const PassVariant*> out;
+    for (int u = 0; u <= (uni ? 1 : 0); ++u)          // staged-tile kernels, then union kernels
+        for (int fit = stratified ? 2 : 0; fit < 3; ++fit)  // exact shape, range of d, any shape
+            for (const PassVariant& v : all) {
+                if (v.fp32 != fp32 || v.uni != u) continue;
+                const int is = v.D > 0 ? 0 : (v.dhi > 0 ? 1 : 2);
+                if (is != fit || (is == 0 && (v.D != d || v.NB != n)) || (is == 1 && (d < v.dlo || d > v.dhi))) continue;
+                out.push_back(&v);
+            }
+    return out;
 }
 
 cudaError_t ensure_smem(const void* fn, size_t bytes)

@@ -229,7 +229,7 @@ cudaError_t launch_union_build(const Params& P, cudaStream_t s)
 
 size_t union_pass_smem(const Params& P, const PassVariant& v, int mode)
 {
-    const int DM = v.D > 0 ? v.D : DMAX;
+    const int DM = v.D > 0 ? v.D : (v.dhi > 0 ? v.dhi : DMAX);
     return (size_t)union_smem_layout(DM, P.d, P.n, mode).bytes;
 }
 
