@@ -32,7 +32,6 @@
 namespace vamp {
 
 constexpr int DMAX = 16;      // largest supported dimension
-constexpr int PASS_THREADS_DEV = 256;  // threads per pass CTA (PASS_THREADS of vamp_internal.h)
 constexpr int MAXMAP = 4;     // mapped coordinates per channel / peak
 constexpr int MAX_BINS = 256; // largest supported bins per axis (table entries are bytes)
 
@@ -255,7 +254,6 @@ template <> struct Prec<double> {
         return __dadd_rn(e0, __dmul_rn(fr, __dsub_rn(e1, e0)));
     }
     static __device__ __forceinline__ double tan_(double v) { return sf_tan(v); }
-    static __device__ __forceinline__ double atan_(double v) { return atan(v); }
     // v^(-1/5) for a normal v > 0 (Newton's method for the inverse fifth
     // root): with v = m 2^E, m in [1, 2), write -E = 5a + r (r in 0..4), so
     // v^(-1/5) = 2^a w^(-1/5) with w = m 2^-r in [1/16, 2).  The seed
@@ -282,12 +280,6 @@ template <> struct Prec<double> {
         }
         return y * __longlong_as_double((long long)(1023 + a) << 52);  // times 2^a
     }
-    // v^0.2 = v (v^(-1/5))^4
-    static __device__ __forceinline__ double pow02(double v)
-    {
-        const double y = rinv5(v), y2 = y * y;
-        return v * (y2 * y2);
-    }
     // v^-0.8 = (v^(-1/5))^4
     static __device__ __forceinline__ double powm08(double v)
     {
@@ -295,7 +287,6 @@ template <> struct Prec<double> {
         return y2 * y2;
     }
     static __device__ __forceinline__ double exp2_(double v) { return exp2(v); }
-    static __device__ __forceinline__ double div(double a, double b) { return a / b; }
     static __device__ __forceinline__ double tiny() { return 2.2250738585072014e-308; }
     // e <= x for the non-negative edges: compare bit patterns (integer pipe)
     static __device__ __forceinline__ bool le(double e, double x)
