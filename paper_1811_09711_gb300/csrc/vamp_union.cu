@@ -16,11 +16,12 @@
 //                   FP32 density 1/(nΔx) of the bin of row (c, k) whose image
 //                   holds it: the largest j <= n-1 with image_j <= U_k[u]
 //                   (bin 0 below the first image), from the lookup block.
-// For the collider (d = 14, K = 64, n = 100) they take 5, 48, 7 and 19 us.  A
-// bitonic sort, two searches per cell and a search per density took 70, 18 and
-// 49; ranking every image in every other channel's row took 49, and a thread
-// filling the cells up to its value's successor 75 to 125, long gaps being
-// filled by one thread.
+// For the collider (d = 14, K = 64, n = 100) they take 5, 22, 7 and 19 us, the
+// first three bounded by latency and the last by writing 23 MB of densities.
+// A bitonic sort, two searches per cell and a search per density took 70, 18
+// and 49; placing every image by a search in its neighbour list at each merge
+// 48, in every other channel's row 49; a thread filling the cells up to its
+// value's successor 75 to 125, long gaps being filled by one thread.
 #include "vamp_union.cuh"
 
 #include <algorithm>
@@ -57,12 +58,10 @@ __global__ void k_union_images(Params P)
 }
 
 constexpr int SORT_THREADS = 1024;
-constexpr int SORT_ILP = 4;
 
 __device__ __forceinline__ int pow2_floor(int v) { return 1 << (31 - __clz(v)); }
 
 // One block per coordinate; dynamic shared memory: the K (n+1) images twice.
-// Shared-memory latency bounds it; four searches per thread are in flight.
 __global__ void __launch_bounds__(SORT_THREADS, 1) k_union_sort(Params P)
 {
     extern __shared__ float sv[];
@@ -90,49 +89,35 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_union_sort(Params P)
         }
     }
     __syncthreads();
-    // Neighbouring lists of w values merge into one: a value's place is its
-    // own index plus the count of the other list's before it, equal ones of
-    // the left list first.
+    // Neighbouring lists of w values merge into one, equal values of the left
+    // list first.  Each thread makes a run of outputs: where the two lists
+    // stand at its start by a search along the diagonal, then value by value.
+    // The runs have odd length, so that a warp's accesses spread over the banks.
+    const int per = ((m + SORT_THREADS - 1) / SORT_THREADS) | 1;
+    const int i0 = min(tid * per, m), i1 = min(i0 + per, m);
     for (int w = n1; w < m; w *= 2) {
-        const int top = pow2_floor(min(w, m));
-        for (int i0 = tid; i0 < m; i0 += SORT_ILP * SORT_THREADS) {
-            float v[SORT_ILP];
-            int at[SORT_ILP], base[SORT_ILP], len[SORT_ILP], lo[SORT_ILP];
-            bool le[SORT_ILP];
-#pragma unroll
-            for (int q = 0; q < SORT_ILP; ++q) {
-                const int i = min(i0 + q * SORT_THREADS, m - 1);
-                const int l = i / w;
-                v[q] = src[i];
-                le[q] = l & 1;
-                base[q] = (l ^ 1) * w;
-                len[q] = max(min(w, m - base[q]), 0);
-                at[q] = i - (le[q] ? w : 0);
-                lo[q] = 0;
+        for (int o = i0; o < i1;) {
+            const int p0 = o / (2 * w) * (2 * w), t = o - p0;
+            const int la = min(w, m - p0), lb = min(w, m - p0 - la), end = min(i1, p0 + la + lb);
+            const float *A = src + p0, *B = A + la;
+            int lo = max(0, t - lb), hi = min(t, la);
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (A[mid] <= B[t - 1 - mid]) lo = mid + 1; else hi = mid;
             }
-            for (int b = top; b; b >>= 1) {
-#pragma unroll
-                for (int q = 0; q < SORT_ILP; ++q) {
-                    const int p = lo[q] + b;
-                    if (p <= len[q]) {
-                        const float y = src[base[q] + p - 1];
-                        if (le[q] ? y <= v[q] : y < v[q]) lo[q] = p;
-                    }
-                }
+            int i = lo, j = t - lo;
+            for (; o < end; ++o) {
+                const bool left = j >= lb || (i < la && !(B[j] < A[i]));
+                dst[o] = left ? A[i] : B[j];
+                if (left) ++i; else ++j;
             }
-#pragma unroll
-            for (int q = 0; q < SORT_ILP; ++q)
-                if (i0 + q * SORT_THREADS < m) dst[at[q] + lo[q]] = v[q];
         }
         __syncthreads();
         float* t = src;
         src = dst;
         dst = t;
     }
-    // distinct values, in order: each thread a contiguous run, block scan of
-    // the run counts
-    const int per = (m + SORT_THREADS - 1) / SORT_THREADS;
-    const int i0 = min(tid * per, m), i1 = min(i0 + per, m);
+    // distinct values, in order: a block scan of the runs' counts
     int cnt = 0;
     for (int i = i0; i < i1; ++i) cnt += (i == 0 || src[i] != src[i - 1]) ? 1 : 0;
     int incl = cnt;
