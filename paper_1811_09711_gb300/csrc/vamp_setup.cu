@@ -360,8 +360,9 @@ cudaError_t upload_setup(const Params& P, const Setup& S, cudaStream_t s, bool b
 // different ones, so that calls of one bin rarely meet at one word (an FP64
 // add in shared memory is a compare-and-swap loop: a d = 4, n = 20 pass went
 // through it 36 times per add with one copy).  Every segment clears and sums
-// all copies, so they are kept below 8 KB: with 32 KB the small passes and the
-// 32-problem batch lost more than they gained (8.65 -> 9.99 ms).
+// the copies that it uses, so the plan keeps them within 16 KB and a segment of
+// few calls takes fewer (vamp_pass.cuh): with 32 KB, all used by every segment,
+// the 32-problem batch went from 8.65 to 9.99 ms.
 TilePlan plan_tiles(size_t S, int K, int dn, size_t fixed, size_t budget)
 {
     const size_t most = 16 * 1024, one = (size_t)dn * 8;

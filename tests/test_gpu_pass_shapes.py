@@ -1,8 +1,8 @@
 """Shapes at which the pass kernels change what they do, against the FP64 oracle.
 
 The staged-tile pass keeps 1 to 32 copies of a segment's d-values in shared
-memory (as many as fit 8 KB, none for a segment with fewer calls than it has
-words to clear), cuts its calls into whole warps, and skips warps without
+memory (as many as fit 16 KB, fewer for a segment with under
+four calls per bin and copy), cuts its calls into whole warps, and skips warps without
 calls.  Sums of FP64 weights that agree with the oracle's to a few 1e-16 per
 term, added in another order: bars 1e-12, as for every FP64 run.
 """
@@ -84,8 +84,8 @@ BW, POW = P.MAP_BW, P.MAP_POW
 
 @pytest.mark.parametrize("d,n,K,calls", [
     (4, 8, 1, 20_000),      # 32 copies (256 words each)
-    (4, 256, 1, 40_000),    # exactly 8 KB with one copy
-    (2, 255, 1, 40_000),    # two copies, ragged
+    (4, 256, 1, 40_000),    # 8 KB with one copy, two fit
+    (2, 255, 1, 40_000),    # four copies, ragged
     (4, 20, 1, 1),          # N_min calls: one warp of one CTA
     (4, 20, 1, 9_728),      # 32 calls for each of 304 CTAs
     (4, 20, 1, 9_729),
