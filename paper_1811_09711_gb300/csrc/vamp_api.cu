@@ -587,10 +587,13 @@ vamp_status vamp_generate(vamp_ctx* c, int64_t n_events, uint32_t gen_id, void* 
         c->g_staging = nullptr; c->g_callidx = nullptr; c->g_counts = nullptr; c->g_offsets = nullptr;
         c->g_cap = 0;
         const int64_t slots = nchunks * chunk;
+        // counts and offsets for the chunks of a kernel with one call per
+        // thread: the context's kernel may change between two calls
+        const int64_t most = (B + vamp::PASS_THREADS - 1) / vamp::PASS_THREADS;
         if (cudaMalloc(&c->g_staging, (size_t)slots * rec) != cudaSuccess ||
             cudaMalloc(&c->g_callidx, (size_t)slots * 4) != cudaSuccess ||
-            cudaMalloc(&c->g_counts, (size_t)nchunks * 4) != cudaSuccess ||
-            cudaMalloc(&c->g_offsets, (size_t)nchunks * 8) != cudaSuccess)
+            cudaMalloc(&c->g_counts, (size_t)most * 4) != cudaSuccess ||
+            cudaMalloc(&c->g_offsets, (size_t)most * 8) != cudaSuccess)
             return fail(c, VAMP_ERR_OOM, "generation staging allocation failed");
         c->g_cap = slots;
     }
