@@ -484,30 +484,31 @@ __device__ void refine_row_dev(const Params& P, int row, int lane, double* ws)
     }
     S = lanes_sum(S);
     if (!(S > 0.0)) return;  // axis kept (R2); lookup blocks unchanged
-    // m_j and its cumulative, 32 bins at a time
-    double M = 0.0;
-    if (lane == 0) C[0] = 0.0;
-    for (int j0 = 0; j0 < n; j0 += 32) {
-        const int j = j0 + lane;
-        double mj = 0.0;
-        if (j < n) {
-            const double r = Dj[j] / S;
-            if (r == 0.0) mj = 0.0;
-            else if (fabs(r - 1.0) < 1e-12) mj = 1.0;
-            else mj = rebin_measure(r, P.grid_alpha);
-            m[j] = mj;
-        }
-        double v = mj;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const double y = __shfl_up_sync(0xffffffffu, v, o);
-            if (lane >= o) v += y;
-        }
-        v += M;
-        if (j < n) C[j + 1] = v;
-        M = __shfl_sync(0xffffffffu, v, 31);
+    for (int j = lane; j < n; j += 32) {
+        const double r = Dj[j] / S;
+        double mj;
+        if (r == 0.0) mj = 0.0;
+        else if (fabs(r - 1.0) < 1e-12) mj = 1.0;
+        else mj = rebin_measure(r, P.grid_alpha);
+        m[j] = mj;
     }
     __syncwarp();
+    // The cumulative of m in bin order, by one lane: C never falls, and stays
+    // the same to the last bit over bins with m = 0, so that the search below
+    // ends in a bin with m > 0.  (A scan by the lanes adds in another order for
+    // each j; its C moves by an ulp over empty bins, and 1 to 10 % of
+    // mirror-symmetric rows with empty bins then divided by their m = 0.)
+    if (lane == 0) {
+        double acc = 0.0;
+        C[0] = 0.0;
+#pragma unroll 8
+        for (int j = 0; j < n; ++j) {
+            acc += m[j];
+            C[j + 1] = acc;
+        }
+    }
+    __syncwarp();
+    const double M = C[n];
     if (!(M > 0.0)) return;
     for (int i = lane; i <= n; i += 32) {
         double ne;
