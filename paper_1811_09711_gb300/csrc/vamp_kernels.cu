@@ -483,7 +483,10 @@ __device__ void refine_row_dev(const Params& P, int row, int lane, double* ws)
         S += w;
     }
     S = lanes_sum(S);
-    if (!(S > 0.0)) return;  // axis kept (R2); lookup blocks unchanged
+    // axis kept (R2), lookup blocks unchanged; likewise where a d-value is
+    // infinite (a weight above 1.3e154 is finite, its square is not), which
+    // leaves no ratio between the bins
+    if (!(S > 0.0 && S < INFINITY)) return;
     for (int j = lane; j < n; j += 32) {
         const double r = Dj[j] / S;
         double mj;

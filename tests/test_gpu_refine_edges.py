@@ -71,3 +71,30 @@ def test_sparse_rows_of_equal_weights(V, n):
         assert np.all(D == np.round(D))
         g.refine_grids()
         check_rows(old, g.get_state()["edges"], D)
+
+
+def huge(d, n, K, smooth=0):
+    """Weights around 1e160: finite, their squares are not."""
+    pr = problem(d, n, K, [[], [P.MAP_BW]], smooth=smooth)
+    return pr.replace(peak_weight=pr.peak_weight * 1e160)
+
+
+@pytest.mark.parametrize("smooth,a", [(0, 1.5), (1, 1.5), (0, 0.5)])
+def test_infinite_d_values_keep_the_axis(V, smooth, a):
+    pr = huge(3, 20, 2, smooth).replace(grid_alpha=a)
+    g = V.Vamp(pr, precision=V.PREC_FP64)
+    old = g.get_state()["edges"]
+    r = g.sample_pass(5000, 0)
+    assert np.isfinite(r.integral) and np.all(np.isinf(g.get_pass()["D"].max(axis=2)))
+    g.refine_grids()
+    assert np.array_equal(g.get_state()["edges"], old)
+    assert g.sample_pass(5000, 0).integral == pytest.approx(r.integral, rel=1e-12)
+
+
+def test_infinite_d_values_keep_the_axis_in_a_batch(V):
+    prs = [huge(3, 20, 2), problem(3, 20, 2, [[], [P.MAP_BW]])]
+    b = V.Batch(prs, precision=V.PREC_FP64, autotune=False)
+    b.iterate([5000, 5000], 0, 1)
+    uniform = np.broadcast_to(np.arange(21) / 20, (2, 3, 21))
+    assert np.array_equal(b.get_state(0)["edges"], uniform)
+    assert not np.array_equal(b.get_state(1)["edges"], uniform)
