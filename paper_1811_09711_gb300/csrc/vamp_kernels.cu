@@ -417,13 +417,23 @@ __global__ void k_derive(Params P, double w_max, int n_hist)
 // ---------------------------------------------------------------------------
 // ((r - 1) / ln r)^a for r in (0, 1): logarithms and powers on 64-bit mantissas
 // (an FP64 log and pow are some 150 operations of the FP64 pipe a bin, half of
-// the rebinning of the collider's 896 rows).  Near 1, where log r is small
-// against its error there, the FP64 log.
+// the rebinning of the collider's 896 rows).  Nothing is rounded to a double
+// before the result, whose error is that rounding's and 2^-58 (grid_alpha 1.5).
+// Above 1/2, which one bin of a row can be, and below a normal number the FP64
+// log.
 __device__ __forceinline__ double rebin_measure(double r, double a)
 {
-    const double lr = r > 0.999 ? log(r) : sf_log2(r) * 0.6931471805599453;
-    const double v = (r - 1.0) / lr;
-    return sf_to_double(sf_norm(sf_exp2(a * sf_log2(v))));
+    Sf num, den;
+    if (r <= 0.5 && r >= 2.3e-308) {
+        bool neg;
+        const Sf x = sf_from_double(r);
+        den = sf_mul(sf_log2(x, neg), Sf{0xb17217f7d1cf79acull, -64});  // -ln r
+        num = Sf{0ull - (x.e > -128 ? x.m >> (-64 - x.e) : 1ull), -64};  // 1 - r
+    } else {
+        den = sf_from_double(-log(r));
+        num = sf_from_double(1.0 - r);
+    }
+    return sf_to_double(sf_pow(sf_norm(sf_mul(num, sf_rcp(sf_norm(den)))), a));
 }
 
 // Doubles of warp scratch of refine_row_dev.
@@ -547,6 +557,17 @@ __global__ void __launch_bounds__(REFINE_WARPS * 32) k_refine(Params P)
 // ---------------------------------------------------------------------------
 // channel weights (Eq. 25 with R5)
 // ---------------------------------------------------------------------------
+// ω^β on 64-bit mantissas (about 2^-57 and the rounding, as long as the power
+// lies within 2^±128); by pow beyond, and where ω or β is not a normal number.
+__device__ __forceinline__ double omega_power(double w, double beta)
+{
+    if (w >= 2.3e-308 && w < INFINITY && fabs(beta) >= 2.3e-308) {
+        const Sf u = sf_pow(sf_from_double(w), beta);
+        if (u.e + 63 >= -128 && u.e + 63 < 128) return sf_to_double(u);
+    }
+    return pow(w, beta);
+}
+
 // Called by every thread of one block, a channel a thread (Acum holds the
 // terms α_c ω_c^β and then the new weights between the sums).
 __device__ void update_alpha_dev(const Params& P)
@@ -559,8 +580,7 @@ __device__ void update_alpha_dev(const Params& P)
         const double a = P.alpha[c], w = omega(c);
         double u = 0.0;
         if (a > 0.0 && P.Nc[c] > 0 && w > 0.0) {
-            // ω^β (pow where ω is beyond a normal number)
-            u = a * (w >= 2.3e-308 && w < INFINITY ? sf_to_double(sf_norm(sf_exp2(P.beta * sf_log2(w)))) : pow(w, P.beta));
+            u = a * omega_power(w, P.beta);
             SU += u;
             MU += a;
         }

@@ -245,31 +245,21 @@ VAMP_HD Sf sf_powm08(double v)
     return sf_norm(Sf{z, -60 - 4 * a});
 }
 
-// 2^x of a finite double (|x| >= 2^20 as 2^±(2^20)), to about 2^-57, normalised: the fraction's
-// leading two bits pick 2^(i/4), the rest goes through the series of 2^t =
-// sum (t ln 2)^k / k! for t in [0, 1/4), whose terms from t^7 on (below 2^-30)
-// are summed in 32 bits.
-VAMP_HD Sf sf_exp2(double x)
+// High 64 bits of a b, exact.
+VAMP_HD uint64_t sf_mulhi_exact(uint64_t a, uint64_t b)
 {
-    const uint64_t b = sf_bits(x);
-    const int ex = (int)((uint32_t)(b >> 52) & 0x7ffu) - 1023;
-    const uint64_t mant = (b << 11) | (1ull << 63);  // |x| = mant 2^(ex - 63)
-    // integer part and 64-bit fraction of |x|
-    int n = 0;
-    uint64_t f;
-    if (ex >= 20) {
-        n = 1 << 20;
-        f = 0ull;
-    } else if (ex >= 0) {
-        n = (int)(mant >> (63 - ex));
-        f = mant << (ex + 1);
-    } else {
-        f = ex >= -64 ? mant >> (-1 - ex) : 0ull;
-    }
-    if (b >> 63) {  // 2^-(n + f) = 2^(-n-1) 2^(1-f)
-        n = f ? -n - 1 : -n;
-        f = 0ull - f;
-    }
+#ifdef __CUDA_ARCH__
+    return __umul64hi(a, b);
+#else
+    return (uint64_t)(((unsigned __int128)a * b) >> 64);
+#endif
+}
+
+// 2^(n + f 2^-64), to about 2^-60, normalised: the fraction's leading two bits
+// pick 2^(i/4), the rest goes through the series of 2^t = sum (t ln 2)^k / k!
+// for t in [0, 1/4), whose terms from t^7 on (below 2^-30) are summed in 32 bits.
+VAMP_HD Sf sf_exp2_fixed(int n, uint64_t f)
+{
     const uint32_t i = (uint32_t)(f >> 62);
     const uint64_t t = f & 0x3fffffffffffffffull;  // Q0.64, below 1/4
     const uint32_t th = (uint32_t)(t >> 32);
@@ -289,24 +279,97 @@ VAMP_HD Sf sf_exp2(double x)
     v = (1ull << 63) + (sf_mulhi(t, v) >> 1);  // 2^t, Q1.63
     const uint64_t k01 = (i & 1u) ? 0x9837f0518db8a96full : 0x8000000000000000ull;
     const uint64_t k23 = (i & 1u) ? 0xd744fccad69d6af4ull : 0xb504f333f9de6484ull;
-    return Sf{sf_mulhi(v, (i & 2u) ? k23 : k01) << 1, n - 63};
+    return Sf{sf_mulhi_exact(v, (i & 2u) ? k23 : k01) << 1, n - 63};
 }
 
-// log2 of a positive normal double: an FP32 logarithm y0 of the significand m
-// in [1, 2), then log2 (m 2^-y0) = d - d^2/2 + ... over ln 2 with d = m 2^-y0 - 1
-// (|d| < 2^-20) from the 64-bit product.  Absolute error about 2^-59 besides
-// the rounding of the sum.
-VAMP_HD double sf_log2(double x)
+// 2^(±m 2^(ex - 63)), m normalised (from 2^20 on as 2^±(2^20)).
+VAMP_HD Sf sf_exp2_parts(bool neg, uint64_t m, int ex)
+{
+    // integer part and 64-bit fraction of the size
+    int n = 0;
+    uint64_t f;
+    if (ex >= 20) {
+        n = 1 << 20;
+        f = 0ull;
+    } else if (ex >= 0) {
+        n = (int)(m >> (63 - ex));
+        f = m << (ex + 1);
+    } else {
+        f = ex >= -64 ? m >> (-1 - ex) : 0ull;
+    }
+    if (neg) {  // 2^-(n + f) = 2^(-n-1) 2^(1-f)
+        n = f ? -n - 1 : -n;
+        f = 0ull - f;
+    }
+    return sf_exp2_fixed(n, f);
+}
+
+// 2^x of a finite double.
+VAMP_HD Sf sf_exp2(double x)
 {
     const uint64_t b = sf_bits(x);
-    const uint64_t m = (b << 11) | (1ull << 63);
-    const int ex = (int)((uint32_t)(b >> 52) & 0x7ffu) - 1023;
-    const double y0 = (double)(sf_lg2f((float)(uint32_t)(m >> 40)) - 23.0f);  // in [0, 1]
-    const Sf t = sf_exp2(-y0);
-    const Sf p = sf_mul(Sf{m, -63}, t);                               // about 1; p.e is -63 or -62
-    const int64_t d = (int64_t)((p.m << (63 + p.e)) - (1ull << 63));  // Q1.63
-    const double dd = (double)d * 0x1p-63;
-    return (y0 + (double)ex) + (dd - 0.5 * dd * dd) * 1.4426950408889634;
+    return sf_exp2_parts(b >> 63, (b << 11) | (1ull << 63), (int)((uint32_t)(b >> 52) & 0x7ffu) - 1023);
+}
+
+// |log2 a| of a normalised number, normalised (zero: m = 0), and its sign: an
+// FP32 logarithm y of the significand s in [1, 2) in 32-bit fixed point, then
+// log2 (s 2^-y) = (d - d^2/2 + ...) / ln 2 of d = s 2^-y - 1 (|d| < 2^-21, the
+// next term below 2^-64).  Integer part and fraction stay apart until the end:
+// error about 2^-60 below 1, relative above.
+VAMP_HD Sf sf_log2(Sf a, bool& neg)
+{
+    const float yf = sf_lg2f((float)(uint32_t)(a.m >> 40) * 0x1p-23f);  // in [0, 1]
+    const uint64_t y = (uint64_t)sf_f2u(yf > 0.f ? yf * 0x1p31f : 0.f) << 1;  // Q0.32, up to 2^32
+    const Sf t = y ? sf_exp2_fixed(-1, 0ull - (y << 32)) : Sf{1ull << 63, -63};  // 2^-y
+    const uint64_t p = sf_mulhi_exact(a.m, t.m);  // s 2^-y 2^(62 + (0 or 1)): t's exponent is -63 or -64
+    const int64_t d = (int64_t)((p << (t.e == -63 ? 1 : 0)) - (1ull << 63));  // Q1.63
+    const int64_t dh = d >> 14;
+    const int64_t c = d - ((dh * dh) >> 36);
+    // c / ln 2 in Q0.64
+#ifdef __CUDA_ARCH__
+    const int64_t r = __mul64hi(c << 20, 0x5c551d94ae0bf85ell) >> 17;
+#else
+    const int64_t r = (int64_t)(((__int128)(c << 20) * 0x5c551d94ae0bf85ell) >> 64) >> 17;
+#endif
+    // n + f 2^-64 = exponent + y + r
+    const uint64_t f0 = y << 32, f1 = f0 + (uint64_t)r;
+    int n = a.e + 63 + (int)(y >> 32) + (r < 0 ? -1 : 0) + (f1 < f0 ? 1 : 0);
+    uint64_t f = f1;
+    neg = n < 0;
+    if (neg) {  // size of a negative number
+        n = f ? -n - 1 : -n;
+        f = 0ull - f;
+    }
+    // normalise (n < 2^31)
+    if (n) {
+#ifdef __CUDA_ARCH__
+        const int z = __clz(n);
+#else
+        const int z = __builtin_clz((unsigned)n);
+#endif
+        return Sf{((uint64_t)(uint32_t)n << (32 + z)) | (f >> (32 - z)), -32 - z};
+    }
+    if (f == 0ull) return Sf{0ull, 0};
+#ifdef __CUDA_ARCH__
+    const int z = __clzll((long long)f);
+#else
+    const int z = __builtin_clzll(f);
+#endif
+    return Sf{f << z, -64 - z};
+}
+
+// a^y of a normalised number and a finite normal double, normalised: the
+// logarithm, the product and its fraction are carried in 64 bits, so that the
+// error is about |y log2 a| 2^-63 and max(1, |y|) 2^-59.
+VAMP_HD Sf sf_pow(Sf a, double y)
+{
+    bool neg;
+    const Sf l = sf_log2(a, neg), b = sf_from_double(y);
+    if (l.m == 0ull) return Sf{1ull << 63, -63};
+    uint64_t m = sf_mulhi_exact(l.m, b.m);
+    int e = l.e + b.e + 64;
+    sf_norm(m, e);
+    return sf_exp2_parts(neg != (sf_bits(y) >> 63 != 0ull), m, e + 63);
 }
 
 // tan of a double |th| < pi/2, to about 2^-58: the ninth convergent of Lambert's

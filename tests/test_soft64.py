@@ -1,0 +1,82 @@
+"""The 64-bit mantissa arithmetic of the FP64 kernels, on the host, against
+arithmetic of 200 bits.
+
+The header is one source for both sides; only the FP32 starting values (an
+approximate instruction on the GPU, the C library here) and the widening
+multiplication are spelled differently.
+"""
+import ctypes as C
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+mp = pytest.importorskip("mpmath")
+mp.mp.prec = 200
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    so = tmp_path_factory.mktemp("soft64") / "soft64.so"
+    subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-o", str(so), os.path.join(HERE, "soft64_host.cpp")],
+                   check=True)
+    return C.CDLL(str(so))
+
+
+def call(lib, name, *ins, sign=False):
+    """The function's results as exact numbers, and their mantissas."""
+    n = len(ins[0])
+    ins = [np.ascontiguousarray(x) for x in ins]
+    m, e, s = np.zeros(n, np.uint64), np.zeros(n, np.int32), np.ones(n, np.int32)
+    args = [*ins, m, e] + ([s] if sign else [])
+    getattr(lib, name)(n, *[a.ctypes.data_as(C.c_void_p) for a in args])
+    return [int(si) * mp.mpf(int(mi)) * mp.mpf(2) ** int(ei) for mi, ei, si in zip(m, e, s)], m
+
+
+def worst(got, want):
+    return max(float(abs(g / w - 1)) for g, w in zip(got, want))
+
+
+def test_exp2(lib):
+    """Ten products and sums of 2^-64 units at a value from 1 to 2, the last
+    one doubled: 2^-59."""
+    rng = np.random.default_rng(1)
+    x = np.concatenate([rng.uniform(-1100, 1100, 3000), rng.uniform(-1, 1, 3000), [0.0, -0.0, 1.0, -1.0, 0.25, 1e-300, -1e-300]])
+    got, m = call(lib, "t_exp2", x)
+    assert np.all(m >> np.uint64(63) == 1)
+    # the argument's own place value: a fraction is cut at 2^-64
+    assert worst(got, [mp.mpf(2) ** mp.mpf(float(v)) for v in x]) < 2.0 ** -59
+
+
+def test_log2(lib):
+    """2^-60 absolute: the power's error, and 2^-63 of larger results."""
+    rng = np.random.default_rng(2)
+    x = np.concatenate([np.exp2(rng.uniform(-1000, 1000, 3000)), rng.uniform(0.5, 2, 3000), 1 + rng.normal(0, 1e-9, 500),
+                        np.exp2(np.arange(-8.0, 9.0)), np.nextafter(np.exp2(np.arange(-8.0, 9.0)), 0)])
+    got, _ = call(lib, "t_log2", x, sign=True)
+    for v, g in zip(x, got):
+        w = mp.log(mp.mpf(float(v)), 2)
+        assert abs(g - w) < 2.0 ** -60 + 2.0 ** -62 * abs(w), v
+
+
+@pytest.mark.parametrize("lo,hi,powers", [
+    (1e-3, 1.0, (1.5,)),          # the measure of the rebinning, at its usual power
+    (1e-3, 1.0, (0.3, 1.0, 3.0)),
+    (1e-10, 1e10, (0.5, 0.25)),   # ω^β, at its usual powers
+    (1e-30, 1e30, (0.5, 1.0, -0.5)),
+    (1e-300, 1e300, (0.125,)),
+])
+def test_pow(lib, lo, hi, powers):
+    """|y log2 x| 2^-62 of the products and the logarithm, 2^-58 of the
+    power; a double's own rounding is 2^-53.  Below that, the result rounded to
+    a double is as near as a library power's."""
+    rng = np.random.default_rng(3)
+    x = np.exp(rng.uniform(np.log(lo), np.log(hi), 3000))
+    for y in powers:
+        got, m = call(lib, "t_pow", x, np.full_like(x, y))
+        assert np.all(m >> np.uint64(63) == 1)
+        bar = 2.0 ** -58 + abs(y) * max(abs(np.log2(lo)), abs(np.log2(hi))) * 2.0 ** -62
+        assert bar < 2.0 ** -53
+        assert worst(got, [mp.mpf(float(v)) ** mp.mpf(y) for v in x]) < bar
