@@ -612,16 +612,31 @@ __global__ void k_update_alpha(Params P)
 // ---------------------------------------------------------------------------
 // generation bookkeeping
 // ---------------------------------------------------------------------------
+constexpr int SMALL_BLOCK = 256;  // most threads of the one-block kernels
+
+// Cumulative α in channel order, by one thread: A_c never falls and stays the
+// same where α_c = 0, so that no call draws a channel that is switched off (in
+// the sums of a scan by lanes such a channel's A_c could lie an ulp higher).
+// Once per generation: K additions from shared memory.
 __global__ void k_gen_prepare(Params P)
 {
-    __shared__ double tmp[33];
+    __shared__ double a[SMALL_BLOCK], sum[SMALL_BLOCK];
+    const int nt = blockDim.x;
     double acc = 0.0;
-    for (int c0 = 0; c0 < P.K; c0 += blockDim.x) {
-        const int c = c0 + (int)threadIdx.x;
-        double tot;
-        const double v = block_scan(c < P.K ? P.alpha[c] : 0.0, tmp, &tot);
-        if (c < P.K) P.Acum[c] = acc + v;
-        acc += tot;
+    for (int c0 = 0; c0 < P.K; c0 += nt) {
+        const int c = c0 + (int)threadIdx.x, m = min(nt, P.K - c0);
+        if (c < P.K) a[threadIdx.x] = P.alpha[c];
+        __syncthreads();
+        if (threadIdx.x == 0) {
+#pragma unroll 8
+            for (int q = 0; q < m; ++q) {
+                acc += a[q];
+                sum[q] = acc;
+            }
+        }
+        __syncthreads();
+        if (c < P.K) P.Acum[c] = sum[threadIdx.x];
+        __syncthreads();
     }
     if (threadIdx.x == 0) P.sc->gen_bmax_bits = 0ull;
 }
@@ -929,7 +944,7 @@ cudaError_t launch_wait_selftest(long long limit, unsigned int* flag, long long*
 // host-side launchers
 // ---------------------------------------------------------------------------
 // Threads of the one-block kernels: a channel a thread up to 256.
-static int small_block(int K) { return std::min(256, (K + 31) / 32 * 32); }
+static int small_block(int K) { return std::min(SMALL_BLOCK, (K + 31) / 32 * 32); }
 
 cudaError_t launch_begin_pass(const Params& P, int64_t N, cudaStream_t s, int clear, int64_t cells)
 {
