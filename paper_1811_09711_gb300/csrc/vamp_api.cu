@@ -315,11 +315,12 @@ vamp_status choose_variant(vamp_ctx* c, int64_t n_calls)
         if (ts != VAMP_OK) return ts;
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
-        // the probe touched the accumulators and the pass scalars (not the
-        // combination history: tuning runs before the first pass)
+        // the probe touched the accumulators, the allocation and the flags at
+        // the head of the scalars; w_max and the history of passes behind them
+        // may come from a restored state
         VAMP_CK(c, cudaMemsetAsync(c->prm.D, 0, (size_t)c->K * c->d * c->n * 8, c->stream));
         VAMP_CK(c, cudaMemsetAsync(c->prm.csum, 0, (size_t)2 * c->K * 8, c->stream));
-        VAMP_CK(c, cudaMemsetAsync(c->prm.sc, 0, HEAD_BYTES, c->stream));
+        VAMP_CK(c, cudaMemsetAsync(c->prm.sc, 0, offsetof(Scalars, wmax_gen), c->stream));
         VAMP_CK(c, cudaStreamSynchronize(c->stream));
         std::lock_guard<std::mutex> lk(g_tune_mu);
         if (!reduced) g_tuned[key] = best;  // a choice made without the union kernels is not kept
