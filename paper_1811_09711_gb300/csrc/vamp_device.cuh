@@ -76,10 +76,6 @@ struct ChanHdr {
 // call folded into two constants.
 template <>
 struct alignas(16) ChanHdr<double> {
-    uint32_t mask;       // bit k: coordinate k is mapped
-    uint32_t kinds;      // byte s: map kind of slot s
-    uint64_t slotpack;   // 4 bits per coordinate: its slot
-    double wz;           // matching peak: weight x Z^-(d - nmap)
     uint32_t slow;       // bit k: some cell of (unmapped) row k overlaps more than two bins
     uint32_t mmask;      // bit k: coordinate k has a Breit-Wigner or power-law map
     double gN;           // Π_BW Γ/A x 0.2^(number of power-law slots): times α the constant of the term of g(p)
@@ -90,7 +86,6 @@ struct alignas(16) ChanHdr<double> {
     double c0[MAXMAP], c1[MAXMAP];    // Breit-Wigner: m, Γ²; power law: δ
     double fw[MAXMAP][3];             // Breit-Wigner: Γ, A, atan(m/Γ)
     float pinvG[MAXMAP], pt0[MAXMAP], pscale[MAXMAP];  // FP32 inverse map to cells: (atan(dp/Γ) + t0) scale; x scale
-    double sp[MAXMAP][SP_N];  // per slot: m, Γ, A, Γ², 1/Γ, Γ/A, 1/A, atan(m/Γ), δ, 1/powN
 };
 static_assert(sizeof(ChanHdr<float>) % 16 == 0 && sizeof(ChanHdr<double>) % 16 == 0, "header not 16-byte sized");
 
@@ -413,6 +408,23 @@ struct Shape {
         return blk + H() + k * R();
     }
 };
+
+// Slot of coordinate k among a channel's Breit-Wigner and power-law maps, -1
+// if it has none.
+__device__ __forceinline__ int map_slot(const ChanHdr<double>& h, int k)
+{
+    for (int s = 0; s < (int)h.nslot; ++s)
+        if ((h.sk[s] & 15) == k) return s;
+    return -1;
+}
+
+// Image φ(x) of a grid edge under slot s, by the forward map's formula.
+__device__ __forceinline__ double edge_image(const ChanHdr<double>& h, int s, double x)
+{
+    if ((h.sk[s] >> 4) == MAP_BW) return h.c0[s] + h.fw[s][0] * Prec<double>::tan_(h.fw[s][1] * x - h.fw[s][2]);
+    const double x2 = x * x, x4 = x2 * x2, v = x4 * x;
+    return v < Prec<double>::tiny() ? Prec<double>::tiny() : v;
+}
 
 // Bin of x in a row whose cells overlap at most two bins: the cell's table
 // entry, plus one if x reaches the next edge.

@@ -318,28 +318,16 @@ __device__ __forceinline__ void derive_row_t(const Params& P, const BlkLayout& L
     // (clamped at 0, the forward map's formula): a bin of x = φ_c^{-1}(p) is
     // the bin whose image holds p, so the FP64 lookups compare p itself; the
     // forward map reads the edges from the master grid
-    int kind = MAP_ID;
-    const double* sp = nullptr;
-    if (sizeof(T) == 8) {
-        const ChanHdr<double>* h = reinterpret_cast<const ChanHdr<double>*>(lk + (size_t)c * L.bytes);
-        if ((h->mask >> k) & 1u) {
-            const int s = (int)((h->slotpack >> (4 * k)) & 0xFu);
-            kind = (h->kinds >> (8 * s)) & 0xff;
-            sp = h->sp[s];
-        }
-    }
-    const bool over_x = sizeof(T) == 8 && kind != MAP_ID;
+    const ChanHdr<T>& h = *reinterpret_cast<const ChanHdr<T>*>(lk + (size_t)c * L.bytes);
+    int slot = -1;
+    if constexpr (sizeof(T) == 8) slot = map_slot(h, k);
+    const bool over_x = slot >= 0;
     const int Lc = 1 << L.lshift;
     for (int j = lane; j <= n; j += 32) {
         const double x = e64[j];
         double v = x;
-        if (kind == MAP_BW) {
-            v = sp[SP_M] + sp[SP_G] * Prec<double>::tan_(sp[SP_A] * v - sp[SP_T0]);
-        } else if (kind == MAP_POW) {
-            const double v2 = v * v, v4 = v2 * v2;
-            v = v4 * v;
-            if (v < Prec<double>::tiny()) v = Prec<double>::tiny();
-        }
+        if constexpr (sizeof(T) == 8)
+            if (over_x) v = edge_image(h, slot, x);
         const T ev = (T)(v > 0.0 ? v : 0.0);
         e[j] = ev;
         // first cell boundary q/L at or above the edge (over x in the FP64 rows

@@ -84,70 +84,74 @@ MapRec<T> make_rec(const vamp_map_desc& r, double weight, double zinv, int d)
     return o;
 }
 
-template <typename T>
-void make_hdr(const vamp_map_desc& r, double weight, double zinv, int d, int lshift, unsigned char* out)
+void make_hdr32(const vamp_map_desc& r, double weight, double zinv, int d, unsigned char* out)
 {
-    ChanHdr<T> h;
+    ChanHdr<float> h;
     std::memset(&h, 0, sizeof h);
-    h.wz = (T)(weight * std::pow(zinv, (double)(d - r.n_mapped)));
+    h.wz = (float)(weight * std::pow(zinv, (double)(d - r.n_mapped)));
     for (int s = 0; s < r.n_mapped; ++s) {
         const int k = r.coord[s];
         h.mask |= 1u << k;
         h.slotpack |= (uint64_t)s << (4 * k);
         h.kinds |= (uint32_t)(r.kind[s] & 0xff) << (8 * s);
-        T* sp = h.sp[s];
+        float* sp = h.sp[s];
         if (r.kind[s] == VAMP_MAP_BW) {
             const double m = r.a[s], G = r.b[s], A = bw_A(m, G);
-            sp[SP_M] = (T)m;
-            sp[SP_G] = (T)G;
-            sp[SP_A] = (T)A;
-            sp[SP_G2] = (T)(G * G);
-            sp[SP_INVG] = (T)(1.0 / G);
-            sp[SP_GINVA] = (T)(G / A);
-            sp[SP_INVA] = (T)(1.0 / A);
-            sp[SP_T0] = (T)std::atan(m / G);
+            sp[SP_M] = (float)m;
+            sp[SP_G] = (float)G;
+            sp[SP_A] = (float)A;
+            sp[SP_G2] = (float)(G * G);
+            sp[SP_INVG] = (float)(1.0 / G);
+            sp[SP_GINVA] = (float)(G / A);
+            sp[SP_INVA] = (float)(1.0 / A);
+            sp[SP_T0] = (float)std::atan(m / G);
         } else if (r.kind[s] == VAMP_MAP_POW) {
-            sp[SP_DEL] = (T)r.b[s];
-            sp[SP_INVPOWN] = (T)pow_invN(r.b[s]);
+            sp[SP_DEL] = (float)r.b[s];
+            sp[SP_INVPOWN] = (float)pow_invN(r.b[s]);
         }
     }
-    if constexpr (sizeof(T) == 8) {
-        // the slots with a factor, and the constants of the channel's terms
-        // (SoftCall); a map whose constants are not finite makes them so too,
-        // and with them the weights, which are then reported
-        h.gN = 1.0;
-        h.fN = h.wz;
-        for (int s = 0; s < r.n_mapped; ++s) {
-            const int kind = r.kind[s], q = (int)h.nslot;
-            if (kind != MAP_BW && kind != MAP_POW) continue;
-            h.mmask |= 1u << r.coord[s];
-            h.sk[q] = (uint8_t)(r.coord[s] | kind << 4);
-            // cells of the row's table per unit of the FP32 inverse map, whose
-            // error (about 2e-6 / A) must stay below the 0.02 cells that the
-            // lookup allows it; 0: the search starts at the first bin
-            const double cells = (double)(1 << lshift);
-            if (kind == MAP_BW) {
-                const double A = h.sp[s][SP_A];
-                h.bw = 1;
-                h.c0[q] = h.sp[s][SP_M];
-                h.c1[q] = h.sp[s][SP_G2];
-                h.fw[q][0] = h.sp[s][SP_G];
-                h.fw[q][1] = A;
-                h.fw[q][2] = h.sp[s][SP_T0];
-                h.gN *= h.sp[s][SP_GINVA];
-                h.fN *= h.sp[s][SP_GINVA];
-                if (!(h.sp[s][SP_G2] >= 2.3e-308)) h.gN = h.fN = NAN;  // Γ² vanishes
-                h.pinvG[q] = (float)h.sp[s][SP_INVG];
-                h.pt0[q] = (float)h.sp[s][SP_T0];
-                h.pscale[q] = A > 0.3 ? (float)(cells / A) : 0.f;
-            } else {
-                h.c0[q] = h.sp[s][SP_DEL];
-                h.gN *= 0.2;
-                h.fN *= h.sp[s][SP_INVPOWN];
-                h.pscale[q] = (float)cells;
-            }
-            ++h.nslot;
+    std::memcpy(out, &h, sizeof h);
+}
+
+// The slots with a factor, and the constants of the channel's terms
+// (SoftCall); a map whose constants are not finite makes them so too, and with
+// them the weights, which are then reported.
+void make_hdr64(const vamp_map_desc& r, double weight, double zinv, int d, int lshift, unsigned char* out)
+{
+    ChanHdr<double> h;
+    std::memset(&h, 0, sizeof h);
+    h.gN = 1.0;
+    h.fN = weight * std::pow(zinv, (double)(d - r.n_mapped));
+    for (int s = 0; s < r.n_mapped; ++s) {
+        const int kind = r.kind[s], q = (int)h.nslot;
+        if (kind != MAP_BW && kind != MAP_POW) continue;
+        h.mmask |= 1u << r.coord[s];
+        h.sk[q] = (uint8_t)(r.coord[s] | kind << 4);
+        // cells of the row's table per unit of the FP32 inverse map, whose
+        // error (about 2e-6 / A) must stay below the 0.02 cells that the
+        // lookup allows it; 0: the search starts at the first bin
+        const double cells = (double)(1 << lshift);
+        if (kind == MAP_BW) {
+            const double m = r.a[s], G = r.b[s], A = bw_A(m, G), t0 = std::atan(m / G);
+            h.bw = 1;
+            h.c0[q] = m;
+            h.c1[q] = G * G;
+            h.fw[q][0] = G;
+            h.fw[q][1] = A;
+            h.fw[q][2] = t0;
+            h.gN *= G / A;
+            h.fN *= G / A;
+            if (!(G * G >= 2.3e-308)) h.gN = h.fN = NAN;  // Γ² vanishes
+            h.pinvG[q] = (float)(1.0 / G);
+            h.pt0[q] = (float)t0;
+            h.pscale[q] = A > 0.3 ? (float)(cells / A) : 0.f;
+        } else {
+            h.c0[q] = r.b[s];
+            h.gN *= 0.2;
+            h.fN *= pow_invN(r.b[s]);
+            h.pscale[q] = (float)cells;
         }
+        ++h.nslot;
     }
     std::memcpy(out, &h, sizeof h);
 }
@@ -257,8 +261,8 @@ bool build_setup(const vamp_config* cfg, Params& pr, Setup& S, std::string& why)
     for (int q = 0; q < K; ++q) {
         // with matching peaks the channel header carries the peak weight too
         const double w = pr.matching ? cfg->peak_weight[q] : 0.0;
-        make_hdr<double>(cfg->channels[q], w, S.zinv, d, pr.lay64.lshift, S.hdr64.data() + (size_t)q * pr.lay64.H);
-        make_hdr<float>(cfg->channels[q], w, S.zinv, d, pr.lay32.lshift, S.hdr32.data() + (size_t)q * pr.lay32.H);
+        make_hdr64(cfg->channels[q], w, S.zinv, d, pr.lay64.lshift, S.hdr64.data() + (size_t)q * pr.lay64.H);
+        make_hdr32(cfg->channels[q], w, S.zinv, d, S.hdr32.data() + (size_t)q * pr.lay32.H);
     }
     S.pk64.assign((size_t)P * sizeof(MapRec<double>), 0);
     S.pk32.assign((size_t)P * sizeof(MapRec<float>), 0);

@@ -39,20 +39,9 @@ __global__ void k_union_images(Params P)
         const int c = (int)((t / n1) % K);
         const int k = (int)(t / ((int64_t)n1 * K));
         const double e = P.edges64[((size_t)c * d + k) * n1 + j];
-        const ChanHdr<double>* h = reinterpret_cast<const ChanHdr<double>*>(P.lk64 + (size_t)c * P.lay64.bytes);
-        double v = e;
-        if ((h->mask >> k) & 1u) {
-            const int s = (int)((h->slotpack >> (4 * k)) & 0xFu);
-            const int kind = (h->kinds >> (8 * s)) & 0xff;
-            const double* sp = h->sp[s];
-            if (kind == MAP_BW) {
-                v = sp[SP_M] + sp[SP_G] * Prec<double>::tan_(sp[SP_A] * e - sp[SP_T0]);
-            } else if (kind == MAP_POW) {
-                const double e2 = e * e, e4 = e2 * e2;
-                v = e4 * e;
-                if (v < Prec<double>::tiny()) v = Prec<double>::tiny();
-            }
-        }
+        const ChanHdr<double>& h = *reinterpret_cast<const ChanHdr<double>*>(P.lk64 + (size_t)c * P.lay64.bytes);
+        const int s = map_slot(h, k);
+        const double v = s >= 0 ? edge_image(h, s, e) : e;
         P.uImg[t] = __double2float_ru(v);  // [k][c][j]
     }
 }
