@@ -78,10 +78,14 @@ template <>
 struct alignas(16) ChanHdr<double> {
     uint32_t slow;       // bit k: some cell of (unmapped) row k overlaps more than two bins
     uint32_t mmask;      // bit k: coordinate k has a Breit-Wigner or power-law map
-    double gN;           // Π_BW Γ/A x 0.2^(number of power-law slots): times α the constant of the term of g(p)
+    double gN;           // Π_BW Γ/A x 0.2^(number of power-law slots), times α the constant of the term of g(p)
     double fN;           // wz Π_BW Γ/A Π_POW 1/powN: the constant of the matching peak
     uint32_t nslot;      // Breit-Wigner and power-law slots
-    uint32_t bw;         // some are Breit-Wigner
+    uint32_t bw;         // 1: some are Breit-Wigner; 2: of widths far from 1
+    // bw = 2: gN and fN are 2^-ge of the above, and the denominators' product
+    // is divided by 2^ge, so that neither leaves the range of a double where
+    // their ratio does not (0 otherwise)
+    int32_t ge;
     uint8_t sk[MAXMAP];  // their coordinate | kind << 4
     double c0[MAXMAP], c1[MAXMAP];    // Breit-Wigner: m, Γ²; power law: δ
     double fw[MAXMAP][3];             // Breit-Wigner: Γ, A, atan(m/Γ)
@@ -734,7 +738,7 @@ __device__ __forceinline__ void soft_forward(const Params& P, const SH& sh, int 
         if (k % 8 == 7 || k == SH::DM - 1) sf_norm(acc, ae);
     }
     const Sf one{1ull << 63, -63};
-    Sf den = one, G = one;
+    Sf den{1ull << 63, -63 - __ldg(&h->ge)}, G = one;
     const int ns = (int)__ldg(&h->nslot);
 #pragma unroll 1
     for (int s = 0; s < ns; ++s) {
@@ -744,13 +748,13 @@ __device__ __forceinline__ void soft_forward(const Params& P, const SH& sh, int 
             const double* sp = h->fw[s];
             const double t = __ldg(sp) * Prec<double>::tan_(__ldg(sp + 1) * x - __ldg(sp + 2));  // p - m, before p is rounded
             const double pk = __ldg(&h->c0[s]) + t, dp = pk - __ldg(&h->c0[s]);
-            den = sf_mul(den, sf_from_double(dp * dp + __ldg(&h->c1[s])));
+            den = sf_mul(den, sf_from_any(dp * dp + __ldg(&h->c1[s])));
             S.p[k] = pk;
         } else {
             const double x2 = x * x, x4 = x2 * x2;
             double pk = x4 * x;
             if (pk < Prec<double>::tiny()) pk = Prec<double>::tiny();
-            G = sf_mul(G, sf_rcp(sf_from_double(x4)));  // (p^(-4/5) from x: p may have been floored)
+            G = sf_mul(G, sf_rcp(sf_from_any(x4)));  // (p^(-4/5) from x: p may have been floored)
             S.p[k] = pk;
         }
     }
@@ -808,6 +812,21 @@ __device__ __forceinline__ float atan_start(float t)
     y = fmaf(y, v, 0.99997723f) * u;
     y = a > 1.f ? 1.57079633f - y : y;
     return copysignf(y, t);
+}
+
+// Product of a channel's Breit-Wigner denominators for widths far from 1 (they
+// need not be normal numbers), divided by 2^ge.  In a loop of its own: tests
+// and powers of two in the loop over all slots took 0.6 of the collider's 53 ms.
+__device__ __forceinline__ Sf far_denominators(const ChanHdr<double>& h, const double* p)
+{
+    Sf den{1ull << 63, -63 - h.ge};
+#pragma unroll 1
+    for (uint32_t s = 0; s < h.nslot; ++s) {
+        if ((h.sk[s] >> 4) != MAP_BW) continue;
+        const double dp = p[h.sk[s] & 15] - h.c0[s];
+        den = sf_mul(den, sf_from_any(dp * dp + h.c1[s]));
+    }
+    return den;
 }
 
 // Channel c' (block in shared or global memory) against one call: its term of
@@ -876,7 +895,10 @@ __device__ __forceinline__ void soft_channel(const Params& P, const SH& sh, cons
         }
     }
     Sf y = one;
-    if (h.bw) y = sf_rcp(sf_norm(den));
+    if (h.bw) {
+        if (h.bw > 1u) den = far_denominators(h, S.p);
+        y = sf_rcp(sf_norm(den));
+    }
     if (with_f && gauss_sum) F = sf_mul(sf_norm(F), sf_exp2(as - S.A));
     gt = ft = 0.0;
     if (lookups) {

@@ -113,15 +113,25 @@ void make_hdr32(const vamp_map_desc& r, double weight, double zinv, int d, unsig
     std::memcpy(out, &h, sizeof h);
 }
 
-// The slots with a factor, and the constants of the channel's terms
-// (SoftCall); a map whose constants are not finite makes them so too, and with
-// them the weights, which are then reported.
+// m 2^e times v, with |m| in [1/2, 1) (m alone where the product is 0 or not finite).
+void scale_by(double& m, int32_t& e, double v)
+{
+    int q = 0;
+    m *= std::isfinite(v) ? std::frexp(v, &q) : v;
+    e += q;
+    if (!std::isfinite(m) || m == 0.0) return;
+    m = std::frexp(m, &q);
+    e += q;
+}
+
+// The slots with a factor, and the constants of the channel's terms (SoftCall).
 void make_hdr64(const vamp_map_desc& r, double weight, double zinv, int d, int lshift, unsigned char* out)
 {
     ChanHdr<double> h;
     std::memset(&h, 0, sizeof h);
-    h.gN = 1.0;
-    h.fN = weight * std::pow(zinv, (double)(d - r.n_mapped));
+    int32_t ge = 0, fe = 0, far = 0;
+    h.gN = h.fN = 1.0;
+    scale_by(h.fN, fe, weight * std::pow(zinv, (double)(d - r.n_mapped)));
     for (int s = 0; s < r.n_mapped; ++s) {
         const int kind = r.kind[s], q = (int)h.nslot;
         if (kind != MAP_BW && kind != MAP_POW) continue;
@@ -134,24 +144,34 @@ void make_hdr64(const vamp_map_desc& r, double weight, double zinv, int d, int l
         if (kind == MAP_BW) {
             const double m = r.a[s], G = r.b[s], A = bw_A(m, G), t0 = std::atan(m / G);
             h.bw = 1;
+            far += std::abs(std::ilogb(G));
             h.c0[q] = m;
             h.c1[q] = G * G;
             h.fw[q][0] = G;
             h.fw[q][1] = A;
             h.fw[q][2] = t0;
-            h.gN *= G / A;
-            h.fN *= G / A;
-            if (!(G * G >= 2.3e-308)) h.gN = h.fN = NAN;  // Γ² vanishes
+            scale_by(h.gN, ge, G / A);
+            scale_by(h.fN, fe, G / A);
             h.pinvG[q] = (float)(1.0 / G);
             h.pt0[q] = (float)t0;
             h.pscale[q] = A > 0.3 ? (float)(cells / A) : 0.f;
         } else {
             h.c0[q] = r.b[s];
-            h.gN *= 0.2;
-            h.fN *= pow_invN(r.b[s]);
+            scale_by(h.gN, ge, 0.2);
+            scale_by(h.fN, fe, pow_invN(r.b[s]));
             h.pscale[q] = (float)cells;
         }
         ++h.nslot;
+    }
+    // without these constants the terms of g(p) and f reach 2^far further than
+    // with them; beyond 2^511 a Γ² is no normal number
+    if (far > 100) {
+        h.bw = 2;
+        h.ge = ge;
+        h.fN = std::ldexp(h.fN, fe - ge);
+    } else {
+        h.gN = std::ldexp(h.gN, ge);
+        h.fN = std::ldexp(h.fN, fe);
     }
     std::memcpy(out, &h, sizeof h);
 }

@@ -98,6 +98,22 @@ VAMP_HD Sf sf_from_double(double x)
     return Sf{(b << 11) | (1ull << 63), (int)((uint32_t)(b >> 52) & 0x7ffu) - SF_BIAS};
 }
 
+// Any finite x >= 0: subnormal numbers as they are, 0 as 2^-65536 (whose
+// reciprocal is beyond a double, as 1 / 0).
+VAMP_HD Sf sf_from_any(double x)
+{
+    const Sf a = sf_from_double(x);
+    if (a.e != -SF_BIAS) return a;
+    const uint64_t m = sf_bits(x) << 11;
+    if (m == 0ull) return Sf{1ull << 63, -65536};
+#ifdef __CUDA_ARCH__
+    const int z = __clzll((long long)m);
+#else
+    const int z = __builtin_clzll(m);
+#endif
+    return Sf{m << z, 1 - SF_BIAS - z};
+}
+
 // Nearest double of a normalised number; 0 below the normal range, infinity above.
 VAMP_HD double sf_to_double(Sf a)
 {
