@@ -257,9 +257,10 @@ bool build_setup(const vamp_config* cfg, Params& pr, Setup& S, std::string& why)
         S.zinv = 1.0 / Z;
         pr.gcen = cc;
         pr.gk2 = M_LOG2E / (2.0 * s * s);
-        // a coordinate's exponent reaches this; packed numbers hold up to 2^960
+        // a coordinate's exponent reaches this (or is no number, which the sum
+        // carries on); packed numbers hold up to 2^960
         const double amax = std::max(cc * cc, (1.0 - cc) * (1.0 - cc)) * pr.gk2;
-        pr.gauss_sum = amax > 900.0;
+        pr.gauss_sum = !(amax <= 900.0);
         pr.gcen_f = (float)cc;
         pr.gk2_f = (float)pr.gk2;
     }

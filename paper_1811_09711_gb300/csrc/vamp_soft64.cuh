@@ -320,11 +320,13 @@ VAMP_HD Sf sf_exp2_parts(bool neg, uint64_t m, int ex)
     return sf_exp2_fixed(n, f);
 }
 
-// 2^x of a finite double.
+// 2^x of a double; beyond a double's range for NaN, of either sign, so that what
+// it enters is not finite.
 VAMP_HD Sf sf_exp2(double x)
 {
     const uint64_t b = sf_bits(x);
-    return sf_exp2_parts(b >> 63, (b << 11) | (1ull << 63), (int)((uint32_t)(b >> 52) & 0x7ffu) - 1023);
+    const bool nan = (b << 1) > 0xffe0000000000000ull;
+    return sf_exp2_parts(!nan && (b >> 63), (b << 11) | (1ull << 63), (int)((uint32_t)(b >> 52) & 0x7ffu) - 1023);
 }
 
 // |log2 a| of a normalised number, normalised (zero: m = 0), and its sign: an

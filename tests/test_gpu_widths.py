@@ -1,4 +1,4 @@
-"""Breit-Wigner widths far from 1, FP64: products of widths, and of the
+"""Constants far from 1, FP64.  Breit-Wigner widths: products of widths, and of the
 denominators (p - m)² + Γ² that divide them, beyond the range of a double where
 their ratio is not; squares of widths that are subnormal or 0.
 
@@ -11,7 +11,7 @@ import os
 import numpy as np
 import pytest
 
-from test_gpu_pass_shapes import BW, problem
+from test_gpu_pass_shapes import BW, POW, problem
 
 pytestmark = pytest.mark.gpu
 NTHREADS = min(16, os.cpu_count() or 4)
@@ -77,3 +77,19 @@ def test_vanishing_square(V, O):
         V.Vamp(pr, precision=V.PREC_FP64).sample_pass(20_000, 0)
     assert err.value.status == V.VAMP_ERR_NUMERIC
     check(V, O, pr, alpha=np.array([0.0, 1.0]))
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("centre,kinds,apart", [
+    (float("nan"), [[]], False),
+    (float("nan"), [[BW], []], False),
+    (-float("nan"), [[BW, POW]], False),
+    (float("nan"), [[BW], []], True),
+    (float("inf"), [[BW], [POW]], False),   # a mapped coordinate's exponent, inf - inf
+])
+def test_gaussian_centre_that_is_no_number(V, precision, centre, kinds, apart):
+    """Accepted at creation; the weights are not finite, and that is reported."""
+    pr = problem(3, 8, 2, kinds, peaks_apart=apart, gauss_centre=centre, gauss_norm=0)
+    with pytest.raises(V.VampError) as err:
+        V.Vamp(pr, precision=precision).sample_pass(20_000, 0)
+    assert err.value.status == V.VAMP_ERR_NUMERIC

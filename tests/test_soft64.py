@@ -50,6 +50,13 @@ def test_exp2(lib):
     assert worst(got, [mp.mpf(2) ** mp.mpf(float(v)) for v in x]) < 2.0 ** -59
 
 
+def test_exp2_beyond(lib):
+    """Infinities and large numbers leave the range of a double on their side, NaN above."""
+    x = np.array([np.inf, 1e300, 2.0 ** 20, np.nan, -np.nan, -np.inf, -1e300])
+    got, _ = call(lib, "t_exp2", x)
+    assert all(g > mp.mpf(2) ** 1024 for g in got[:5]) and all(g < mp.mpf(2) ** -1100 for g in got[5:])
+
+
 def test_log2(lib):
     """2^-60 absolute: the power's error, and 2^-63 of larger results."""
     rng = np.random.default_rng(2)
