@@ -789,7 +789,9 @@ __device__ __forceinline__ void soft_forward(const Params& P, const SH& sh, int 
 }
 
 // Largest j' in [j, n] with e[j'] <= x, for e[j] <= x: three edges at a time,
-// since a search from the right cell seldom goes further.
+// since a search from the right cell seldom goes further.  (Doubling steps
+// after the first three cost 2 to 4 % of every pass, collider 52.9 -> 54.0 ms, for 4 %
+// of a pass over rows with 52 edges in a cell.)
 __device__ __forceinline__ int soft_search(const double* e, int j, int n, double x)
 {
     for (;;) {

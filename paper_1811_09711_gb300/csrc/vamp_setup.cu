@@ -137,9 +137,11 @@ void make_hdr64(const vamp_map_desc& r, double weight, double zinv, int d, int l
         if (kind != MAP_BW && kind != MAP_POW) continue;
         h.mmask |= 1u << r.coord[s];
         h.sk[q] = (uint8_t)(r.coord[s] | kind << 4);
-        // cells of the row's table per unit of the FP32 inverse map, whose
-        // error (about 2e-6 / A) must stay below the 0.02 cells that the
-        // lookup allows it; 0: the search starts at the first bin
+        // cells of the row's table per unit of the FP32 inverse map.  A search
+        // starts 0.02 cells before it, more than its error (2.2e-6 of the
+        // angle, and 2.4e-5 of a small one) above A = 0.3; below, that error is
+        // taken off as well (d = 8, n = 256, two wide or outlying maps a
+        // channel, 1e6 calls: 553 us; from bin 0 on 1 640)
         const double cells = (double)(1 << lshift);
         if (kind == MAP_BW) {
             const double m = r.a[s], G = r.b[s], A = bw_A(m, G), t0 = std::atan(m / G);
@@ -153,8 +155,9 @@ void make_hdr64(const vamp_map_desc& r, double weight, double zinv, int d, int l
             scale_by(h.gN, ge, G / A);
             scale_by(h.fN, fe, G / A);
             h.pinvG[q] = (float)(1.0 / G);
-            h.pt0[q] = (float)t0;
-            h.pscale[q] = A > 0.3 ? (float)(cells / A) : 0.f;
+            const double tmax = std::max(std::fabs(m), std::fabs(1.0 - m)) / G;
+            h.pt0[q] = (float)(A > 0.3 ? t0 : t0 - std::min(2.5e-6, 3e-5 * tmax));
+            h.pscale[q] = (float)(cells / A);
         } else {
             h.c0[q] = r.b[s];
             scale_by(h.gN, ge, 0.2);
