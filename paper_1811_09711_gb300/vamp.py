@@ -214,14 +214,18 @@ assert _MAP_DTYPE.itemsize == C.sizeof(MapDesc) and all(
 
 def _map_array(ms) -> C.Array:
     """The maps as an array of MapDesc, filled a field at a time (a slot at a
-    time took 45 us for six channels and six peaks)."""
+    time took 45 us for six channels and six peaks).  Rows and slots beyond the
+    maps' are ignored; fewer are an IndexError."""
     k = len(ms)
     if k == 0:
         return (MapDesc * 0)()
     rec = np.zeros(k, _MAP_DTYPE)
     rec["n_mapped"] = ms.n_mapped
     for f in ("coord", "kind", "a", "b"):
-        rec[f] = getattr(ms, f)[:, :4]
+        v = getattr(ms, f)
+        if v.shape[0] < k or v.shape[1] < 4:
+            raise IndexError(f"{f} must have 4 slots for each of {k} maps, not shape {v.shape}")
+        rec[f] = v[:k, :4]
     return (MapDesc * k).from_buffer(rec)
 
 
