@@ -300,10 +300,11 @@ vamp_status choose_variant(vamp_ctx* c, int64_t n_calls)
             return VAMP_OK;
         };
         // The two families round differently at bin edges (the union pass
-        // decides a bin exactly for its FP32 p), so which one a problem gets
-        // is settled between their exact-shape and any-shape kernels; the
-        // kernels of a range of d then compete within that family, and do not
-        // move a problem from the more exact one to the other by being faster.
+        // decides a bin exactly for its FP32 p).  Which one a problem gets is
+        // settled between their exact-shape and any-shape kernels, the only
+        // ones there were at first: a problem stays in the family it has been
+        // in, with its bins, and the kernels of a range of d only compete
+        // within it, even where one of the other family would be faster.
         vamp_status ts;
         if (any_uni && !reduced) {
             ts = contest([](const PassVariant* v) { return v->dhi == 0; });

@@ -6,12 +6,17 @@
 // channel loop is products all the way: d bin densities, the Jacobians, the
 // peak's factors.  A product of two 64-bit mantissas is three 32 x 32 -> 64
 // multiplies and a few adds, so a factor costs about eight issue slots
-// instead of the 75 its DMUL occupies, and truncates at 2^-62 instead of
-// rounding at 2^-53.
+// instead of the 75 its DMUL occupies; it is short by less than 2^-60 instead
+// of rounded at 2^-53.
 //
 // A number is m 2^e with m > 0.  "Normalised" means bit 63 of m is set.
 // Products of normalised numbers are not renormalised at once: each loses at
-// most one leading bit, so four products in a row keep 60 bits.
+// most one leading bit.  The kernels chain eight at most, which are short of
+// the true product by less than 2^-52.4 together (largest seen on the GPU:
+// 2^-53.4 for mantissas spread over 1 to 2, 2^-52.8 for mantissas below 1.01;
+// eight products of doubles: 2^-50.9 and 2^-50.5, to either side).
+//
+// The errors below are the largest seen on the GPU over each function's range.
 //
 // A packed number (one 64-bit word, the form of the density rows and of the
 // per-call tables) is the double's 53-bit significand in the high bits and its
@@ -211,7 +216,7 @@ VAMP_HD int64_t sf_scale(uint32_t c, int64_t a, int sh)
     return (hi << (32 - sh)) + (int64_t)(lo >> sh);
 }
 
-// 1 / a of a normalised number, to about 2^-61: an FP32 reciprocal y0 of x =
+// 1 / a of a normalised number, to 2^-60.7: an FP32 reciprocal y0 of x =
 // m 2^-64 in [1/2, 1), then one step of third order (Householder's method),
 // y = y0 (1 + r + r^2) with r = 1 - x y0 taken in 63-bit fixed point (|r| <=
 // 2^-22, so the next term is below 2^-66).
@@ -227,7 +232,7 @@ VAMP_HD Sf sf_rcp(Sf a)
     return Sf{y, -127 - a.e};
 }
 
-// v^(-4/5) of a positive normal double, normalised, to about 2^-57.  With v = X
+// v^(-4/5) of a positive normal double, normalised, to 2^-55.  With v = X
 // 2^(5a), X in [2^-4, 2): an FP32 seed s of X^(-1/5) in (0.87, 1.75), s^2, s^4
 // and s^5 in fixed point, the residual r = 1 - X s^5 (|r| <= 2^-20), and the
 // binomial series (1 - r)^(-4/5) = 1 + (4/5) r + (18/25) r^2 + ... cut after r^2:
@@ -271,7 +276,7 @@ VAMP_HD uint64_t sf_mulhi_exact(uint64_t a, uint64_t b)
 #endif
 }
 
-// 2^(n + f 2^-64), to about 2^-60, normalised: the fraction's leading two bits
+// 2^(n + f 2^-64), to 2^-60, normalised: the fraction's leading two bits
 // pick 2^(i/4), the rest goes through the series of 2^t = sum (t ln 2)^k / k!
 // for t in [0, 1/4), whose terms from t^7 on (below 2^-30) are summed in 32 bits.
 VAMP_HD Sf sf_exp2_fixed(int n, uint64_t f)

@@ -87,3 +87,62 @@ def test_pow(lib, lo, hi, powers):
         bar = 2.0 ** -58 + abs(y) * max(abs(np.log2(lo)), abs(np.log2(hi))) * 2.0 ** -62
         assert bar < 2.0 ** -53
         assert worst(got, [mp.mpf(float(v)) ** mp.mpf(y) for v in x]) < bar
+
+
+@pytest.mark.parametrize("top", [2.0, 1.01])
+def test_eight_products(lib, top):
+    """The k-th product has lost at most k leading bits and is short by three
+    units at most: together less than 3 2^-63 (2 + 4 + ... + 2^8) < 2^-52.4."""
+    rng = np.random.default_rng(4)
+    x, y = rng.uniform(1, top, 4000), rng.uniform(1, top, 4000)
+    got, m = call(lib, "t_products", x, y)
+    assert np.all(m >> np.uint64(63) == 1)
+    off = [float(g / (mp.mpf(float(a)) ** 4 * mp.mpf(float(b)) ** 4) - 1) for g, a, b in zip(got, x, y)]
+    assert max(off) <= 0 and min(off) > -(2.0 ** -52.4)
+
+
+def test_rcp(lib):
+    """Eight units of 2^-63."""
+    x = np.concatenate([np.exp(np.random.default_rng(5).uniform(-700, 700, 4000)), np.exp2(np.arange(-9.0, 9.0)),
+                        np.nextafter(np.exp2(np.arange(-9.0, 9.0)), 0)])
+    got, m = call(lib, "t_rcp", x)
+    assert np.all(m >> np.uint64(63) == 1)
+    assert worst(got, [1 / mp.mpf(float(v)) for v in x]) < 2.0 ** -60
+
+
+def test_rcp_of_subnormal_numbers_and_zero(lib):
+    x = np.concatenate([np.exp2(np.random.default_rng(6).uniform(-1074, -1021, 500)), [5e-324, 2.2250738585072014e-308, 1.0]])
+    got, _ = call(lib, "t_any_rcp", x)
+    assert worst(got, [1 / mp.mpf(float(v)) for v in x]) < 2.0 ** -60
+    assert call(lib, "t_any_rcp", np.zeros(1))[0][0] > mp.mpf(2) ** 60000
+
+
+def test_powm08(lib):
+    """About 30 units of 2^-60: s^4 and its products are fixed-point numbers of 59 to 62 places."""
+    rng = np.random.default_rng(7)
+    x = np.concatenate([np.exp(rng.uniform(-20, 1, 3000)), np.exp(rng.uniform(-708, 0, 3000)), [2.2250738585072014e-308, 1.0]])
+    got, m = call(lib, "t_powm08", x)
+    assert np.all(m >> np.uint64(63) == 1)
+    assert worst(got, [mp.mpf(float(v)) ** (mp.mpf(-4) / 5) for v in x]) < 2.0 ** -55
+
+
+def doubles(lib, name, *ins):
+    r = np.zeros(len(ins[0]))
+    getattr(lib, name)(len(r), *[np.ascontiguousarray(a).ctypes.data_as(C.c_void_p) for a in ins],
+                       r.ctypes.data_as(C.c_void_p))
+    return [mp.mpf(float(v)) for v in r]
+
+
+def test_tan(lib):
+    """Half a unit of the result and 2^-58."""
+    rng = np.random.default_rng(8)
+    x = np.concatenate([rng.uniform(-np.pi / 2, np.pi / 2, 3000), np.pi / 2 - 10.0 ** rng.uniform(-15, 0, 3000),
+                        10.0 ** rng.uniform(-300, 0, 500), [np.pi / 4, np.nextafter(np.pi / 4, 0), np.pi / 2]])
+    assert worst(doubles(lib, "t_tan", x), [mp.tan(mp.mpf(float(v))) for v in x]) < 2.0 ** -53 + 2.0 ** -58
+    assert doubles(lib, "t_tan", np.zeros(1)) == [0]
+
+
+def test_div(lib):
+    rng = np.random.default_rng(9)
+    x, y = rng.normal(0, 1, 4000), np.exp(rng.uniform(-300, 300, 4000))
+    assert worst(doubles(lib, "t_div", x, y), [mp.mpf(float(a)) / mp.mpf(float(b)) for a, b in zip(x, y)]) < 2.0 ** -53 + 2.0 ** -59
